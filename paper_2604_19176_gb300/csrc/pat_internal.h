@@ -46,7 +46,8 @@ constexpr int kQueueStride = 32;
 // Per-instance descriptor (device resident, read by every kernel).
 struct InstDev {
     int32_t n, n_det, n_t, n_r;
-    int32_t K, c0, det_off, pad1;
+    int32_t K, c0, det_off;
+    int32_t tile_off;              // first of the instance's 32 x 8 pixel tiles (img_tiles; row by row)
     float delta, inv_delta, dphi, inv_dphi;
     float inv_K, pad0;
     int32_t n_slots, nmb;          // forward partial slots; radius blocks per detector

@@ -688,11 +688,12 @@ pat_status_t build_plan(Plan& P, const pat_geometry_t* geoms, int n_inst, const 
     std::vector<ImgTile> itiles;
     int64_t time_macs = 0;
     for (int i = 0; i < n_inst; ++i) {
-        const InstDev& d = inst[i];
+        InstDev& d = inst[i];
         for (int j0 = 0; j0 < d.n_det; j0 += kAbelJ) {
             for (int k0 = 0; k0 < d.n_t; k0 += kAbelX) fwd_tiles.push_back({i, j0, k0, 0});
             for (int m0 = 0; m0 < d.n_r; m0 += kAbelX) adj_tiles.push_back({i, j0, m0, 0});
         }
+        d.tile_off = (int32_t)itiles.size();
         for (int y0 = 0; y0 < d.n; y0 += 8)
             for (int x0 = 0; x0 < d.n; x0 += 32) itiles.push_back({i, x0, y0, 0});
         // nonzeros of P: rows kk have m <= kk + 2 (kk = k - 1)
