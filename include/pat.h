@@ -104,8 +104,10 @@ typedef struct {
     int32_t q_piece;     /* max angular nodes per work unit (multiple of 4); 0 = auto        */
     int32_t band_rows;   /* max pixel rows of a circular-mean tile; 0 = auto                 */
     int32_t adj_groups;  /* detector groups of the adjoint gather, 1..16; 0 = auto           */
-    int32_t adj_mode;    /* adjoint gather: 0 = auto (4 if it fits the list budget, else 1,   */
-                         /*   else 3, else 2); 1 = per-cell sample code lists built at        */
+    int32_t adj_mode;    /* adjoint gather: 0 = auto (windowed code lists where adj_groups    */
+                         /*   and adj_jblock are 0 too, a 16-pixel patch's radii fit the      */
+                         /*   staged tables and the codes the list budget; else 4 if it fits  */
+                         /*   the budget, else 1, else 3, else 2); 1 = per-cell sample code lists built at        */
                          /*   creation (device memory ~4 B per sample); 2 = enumerate on      */
                          /*   every call (no list memory); 3 = per-cell fraction lists built  */
                          /*   at creation (~12 B per sample: Mbar index and the FP32 bilinear */
@@ -146,7 +148,8 @@ typedef struct {
     int32_t tile_cols;       /* widest circular-mean tile (pixels); band_rows the tallest */
     int32_t time_pair;       /* 1 = the steps run the fused time stage, 0 = separate      */
     int32_t adj_jblock;      /* detectors per aligned block of the code lists (0: none)   */
-    int32_t reserved;
+    int32_t adj_windows;     /* 1 = the code lists are in windowed form (adj_mode then    */
+                             /*   gives the form that the geometry's codes would take)    */
 } pat_plan_info_t;
 
 /*

@@ -58,7 +58,7 @@ class PatPlanInfo(ctypes.Structure):
         ("adj_groups", ctypes.c_int32), ("bands_max", ctypes.c_int32), ("adj_mode", ctypes.c_int32),
         ("list_bytes", ctypes.c_int64), ("abel_split_fwd", ctypes.c_int32), ("abel_split_adj", ctypes.c_int32),
         ("tile_cols", ctypes.c_int32), ("time_pair", ctypes.c_int32), ("adj_jblock", ctypes.c_int32),
-        ("reserved", ctypes.c_int32),
+        ("adj_windows", ctypes.c_int32),
     ]
 
 

@@ -69,6 +69,12 @@ __device__ __forceinline__ unsigned long long f2_add(unsigned long long a, unsig
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
     return d;
 }
+__device__ __forceinline__ unsigned long long f2_mul(unsigned long long a, unsigned long long b)
+{
+    unsigned long long d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
 __device__ __forceinline__ unsigned long long f2_add_rd(unsigned long long a, unsigned long long b)
 {
     unsigned long long d;
@@ -157,6 +163,49 @@ __device__ __forceinline__ float corner_sum(const float4* __restrict__ z, size_t
     return s;
 }
 
+// The same from the windowed lists' pixel sums: pixel (px, py) is in the core
+// of one 8 x 8 patch and, on a patch's first column or row, also in the
+// right column or top row of the patches before it.
+__device__ __forceinline__ float window_sum(const DevPlan& dp, const InstDev& in, int img, int px, int py)
+{
+    const int sx = px + 1, sy = py + 1;   // cell (px, py)'s index; it is the pixel's own corner 00
+    const int lx = sx & (kWinCells - 1), ly = sy & (kWinCells - 1);
+    const int patch = (sy / kWinCells) * in.win_px + sx / kWinCells;
+    const float* z = dp.win_z + (size_t)(in.win_tile0 + img) * kWinTile;
+    auto at = [&](int p, int o) { return __ldg(z + (size_t)p * (in.win_nimg * kWinTile) + o); };
+    float s = at(patch, ly * kWinCells + lx);
+    if (lx == 0) s += at(patch - 1, 64 + ly);
+    if (ly == 0) s += at(patch - in.win_px, 73 + lx);
+    if (lx == 0 && ly == 0) s += at(patch - in.win_px - 1, 64 + kWinCells);
+    return s;
+}
+
+// Adjoint value of pixel (px, py) of an instance before the 1/K, from
+// whichever cell sums the plan's gather writes.
+__device__ __forceinline__ float adj_pixel(const DevPlan& dp, const InstDev& in, int px, int py)
+{
+    if (dp.n_win_vecs > 0) {
+        // image s at the point that the symmetry's s-th map takes to (px, py)
+        float s = window_sum(dp, in, in.win_img, px, py);
+        const int rx = in.n - 1 - px, ry = in.n - 1 - py;
+        switch (in.win_sym) {
+        case kSymMirrorY: return s + window_sum(dp, in, in.win_img + 1, px, ry);
+        case kSymMirrorX: return s + window_sum(dp, in, in.win_img + 1, rx, py);
+        case kSymDiag: return s + window_sum(dp, in, in.win_img + 1, py, px);
+        case kSymAnti: return s + window_sum(dp, in, in.win_img + 1, ry, rx);
+        case kSymHalf: return s + window_sum(dp, in, in.win_img + 1, rx, ry);
+        case kSymQuarter:   // s quarter turns (x, y) -> (-y, x) taken back
+            s += window_sum(dp, in, in.win_img + 1, py, rx);
+            s += window_sum(dp, in, in.win_img + 2, rx, ry);
+            return s + window_sum(dp, in, in.win_img + 3, ry, px);
+        default: return s;
+        }
+    }
+    const int w = in.n + 1;   // cell (cx, cy) is stored at (cy + 1) * w + (cx + 1)
+    return corner_sum(dp.zbuf + in.z_off, (size_t)w * w, dp.adj_groups, (size_t)(py + 1) * w + px + 1,
+                      (size_t)(py + 1) * w + px, (size_t)py * w + px + 1, (size_t)py * w + px);
+}
+
 // ---------------------------------------------------------------------------
 // TMA (bulk async copy) and mbarrier wrappers
 // ---------------------------------------------------------------------------
@@ -236,6 +285,15 @@ __device__ __forceinline__ void prefetch_l2(const void* src, uint32_t bytes)
 __device__ __forceinline__ void cp_async16(void* dst, const void* src)
 {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+// The same through L1 (for sources that other warps of the SM read too), 16 and 4 bytes.
+__device__ __forceinline__ void cp_async16_l1(void* dst, const void* src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async4_l1(void* dst, const void* src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
 }
 // 4-byte asynchronous copy that writes zero when !valid (nothing is read then).
 __device__ __forceinline__ void cp_async4_zfill(void* dst, const void* src, bool valid)

@@ -498,12 +498,7 @@ __global__ void __launch_bounds__(256) k_adj_combine(DevPlan dp, T* __restrict__
     const int n = in.n;
     const int px = t.x0 + (threadIdx.x & 31), py = t.y0 + (threadIdx.x >> 5);
     if (px >= n || py >= n) return;
-    const int w = n + 1;
-    const float4* z = dp.zbuf + in.z_off;
-    const int groups = dp.adj_groups;
-    // cell (cx, cy) is stored at (cy + 1) * w + (cx + 1)
-    const float s = corner_sum(z, (size_t)w * w, groups, (size_t)(py + 1) * w + px + 1, (size_t)(py + 1) * w + px,
-                               (size_t)py * w + px + 1, (size_t)py * w + px);
+    const float s = adj_pixel(dp, in, px, py);
     const float val = s * in.inv_K;
     if constexpr (sizeof(T) == 4) fout[in.f_off + (size_t)py * n + px] = val;
     else fout[in.f_off + (size_t)py * n + px] = __float2bfloat16(val);
@@ -573,6 +568,7 @@ cudaError_t launch_fill_u32(uint32_t* p, int64_t n, uint32_t v, cudaStream_t st)
 
 cudaError_t launch_adjoint_cells(const DevPlan& dp, cudaStream_t st)
 {
+    if (dp.n_win_vecs > 0) return launch_adj_win(dp, st);
     if (dp.adj_mode == 1 || dp.adj_mode == 3 || dp.adj_mode == 4) {
         if (dp.n_list_items == 0) return cudaSuccess;   // (cell_blocks x 8 warps run the items)
         if (dp.adj_mode == 3) return launch_pdl(k_adj_list<1>, dim3(dp.cell_blocks), dim3(256), 0, st, 1, dp);

@@ -98,6 +98,20 @@ cudaError_t launch_adj_frac_build(const DevPlan& dp, int inst_idx, int n, int32_
 cudaError_t launch_adj_seg(const DevPlan& dp, int inst_idx, int n, bool pairs, int jblock, int nblk, int32_t* seg,
                            const int64_t* pbase, uint32_t* out, cudaStream_t st);
 
+// Windowed lists (windows.cu): the gather, and the steps of list building
+// (windows of every detector and patch; their cut into blocks, counting when
+// blocks == nullptr; staging records; codes, counting when codes == nullptr).
+cudaError_t launch_adj_win(const DevPlan& dp, cudaStream_t st);
+int adj_win_blocks_per_sm(int nb);
+cudaError_t launch_win_windows(const DevPlan& dp, int inst_idx, int n_det, double delta, int patches, int4* win,
+                               cudaStream_t st);
+cudaError_t launch_win_part(const DevPlan& dp, int inst_idx, int patches, int max_rays, int max_slots, int max_longest,
+                            const int4* win, int4* cnt, WinBlock* blocks, WinSub* subs, int32_t* err, cudaStream_t st);
+cudaError_t launch_win_recs(const DevPlan& dp, int inst_idx, int n_blocks, const WinBlock* blocks, const WinSub* subs,
+                            uint2* rayrec, uint32_t* slotrec, cudaStream_t st);
+cudaError_t launch_win_lists(const DevPlan& dp, int inst_idx, int n_blocks, WinBlock* blocks, const WinSub* subs,
+                             uint2* codes, cudaStream_t st);
+
 // p[0 .. n) = v
 cudaError_t launch_fill_u32(uint32_t* p, int64_t n, uint32_t v, cudaStream_t st);
 

@@ -151,10 +151,7 @@ __global__ void __launch_bounds__(256) k_tv_update(DevPlan dp, const float* __re
     float d2 = 0.f, n2 = 0.f;
     if (i < n && j < n) {
         // A^T r at pixel (j, i): corner sums of cells (j,i), (j-1,i), (j,i-1), (j-1,i-1)
-        const int w = n + 1;
-        const float4* z = dp.zbuf + in.z_off;
-        const float s = corner_sum(z, (size_t)w * w, dp.adj_groups, (size_t)(i + 1) * w + j + 1,
-                                   (size_t)(i + 1) * w + j, (size_t)i * w + j + 1, (size_t)i * w + j);
+        const float s = adj_pixel(dp, in, j, i);
         const float adj = s * in.inv_K;
         const float eps2 = eps * eps;
         float dx, dy;
@@ -239,10 +236,7 @@ __global__ void __launch_bounds__(256) k_pdhg_primal(DevPlan dp, float* __restri
     const int j = t.x0 + (threadIdx.x & 31), i = t.y0 + (threadIdx.x >> 5);
     float d2 = 0.f, n2 = 0.f, s1 = 0.f;
     if (i < n && j < n) {
-        const int w = n + 1;
-        const float4* z = dp.zbuf + in.z_off;
-        const float s = corner_sum(z, (size_t)w * w, dp.adj_groups, (size_t)(i + 1) * w + j + 1,
-                                   (size_t)(i + 1) * w + j, (size_t)i * w + j + 1, (size_t)i * w + j);
+        const float s = adj_pixel(dp, in, j, i);
         const size_t idx = in.f_off + (size_t)i * n + j;
         // grad^T p: the differences that pixel (j, i) enters with +1 (from the
         // left / upper neighbour) and -1 (its own, unless on the last column / row)

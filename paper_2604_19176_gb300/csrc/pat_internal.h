@@ -67,6 +67,12 @@ struct InstDev {
     int32_t m_pitch;               // row pitch of M and Mbar: a power of two > n_r (the columns from
                                    //   n_r on stay zero), so a list code's low bits are j * m_pitch + m
     int32_t patches_x;             // adjoint lists: 8 x 4 cell patches per row of cells
+    int32_t win_px;                // windowed lists: 8 x 8 cell patches per row of cells
+    int32_t win_img, win_nimg;     // windowed lists: this instance's first image in its group, and the group's images
+    int32_t win_tile0;             // windowed lists: the group's first pixel-sum tile (WinGroup::tile0)
+    int32_t win_sym;               // windowed lists: the geometry's symmetry (WinSym), its listed detectors and
+    int32_t win_ndet, pad1;        //   images per instance (n_det = win_ndet x the symmetry's order)
+    int64_t win_ray_off;           // windowed lists: offset of the instance's fixed-point directions
 };
 
 // Circular-mean work unit: radii [m0, m0 + m_lanes) of detector j, angles
@@ -148,6 +154,83 @@ struct ListItem {
     int32_t nk, inst, group, x0, y0, pad;
 };
 
+// ---- windowed lists (windows.cu) ------------------------------------------
+constexpr int kWinCells = 8;       // a patch is 8 x 8 cells, patch (0, 0) at cell (-1, -1); one warp works on it
+constexpr int kWinThreads = 128;   // 4 warps, each on its own
+constexpr int kWinPixels = 81;     // 9 x 9 pixels that the cells of a patch touch: the 8 x 8 core, the right column
+                                   //   from the bottom (9), the top row (8)
+constexpr int kWinTile = 96;       // floats of one patch's pixel sums (whole 128-byte lines)
+// Most rays and radii staged per block for groups of nb images (radius slots
+// 0 .. 7 hold zeros); lists of several images are the same for two and four.
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+constexpr int win_rays(int) { return 192; }
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+constexpr int win_slots(int nb) { return nb == 1 ? 1280 : nb == 2 ? 640 : 576; }
+
+// Block of consecutive detector windows of one patch: what a warp stages at
+// once.  Blocks of a template are numbered in patch order, and their staging
+// records and codes follow one another in that order.  The gather reads each
+// block's head, uint4 (patch, n_rays | n_slots << 16, the halves' list lengths).
+struct WinBlock {
+    int32_t patch;
+    uint16_t n_rays, n_slots;      // staged rays (multiple of 4) and radii (multiple of 8, without the zeros)
+    uint32_t ray_rec, slot_rec;    // first staging records (win_rays: 4 rays each; win_slots: 8 radii each)
+    uint2 half[2];                 // lower and upper 8 x 4 cells: first code vector, pair | single vectors << 16
+    uint32_t sub0, n_sub;          // its sub-windows
+};
+
+// Rays q0 .. q0 + nq - 1 (mod K) and radii m0 .. m0 + nm - 1 of detector j,
+// staged from ray slot ray0 and radius slot slot0 (list building only).
+struct WinSub {
+    int32_t j, q0, nq, m0, nm;
+    uint16_t ray0, slot0;
+};
+
+// Symmetry of a geometry: maps of the square that take its detectors to its
+// detectors and its angles to its angles.  Lists are built for the first
+// n_det / order detectors only; image s of an instance gathers the weights of
+// those detectors' s-th copies, and pixel x of the result adds image s at the
+// point that the s-th map takes to x.
+enum WinSym : int32_t {
+    kSymNone = 0,    // order 1
+    kSymMirrorY,     // order 2, (x, y) -> (x, -y): detector j -> n_det - 1 - j
+    kSymMirrorX,     //          (x, y) -> (-x, y)
+    kSymDiag,        //          (x, y) -> (y, x)
+    kSymAnti,        //          (x, y) -> (-y, -x)
+    kSymHalf,        // order 2, half turn: detector j -> j + n_det / 2
+    kSymQuarter      // order 4, quarter turns: detector j -> j + s n_det / 4
+};
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+inline int win_sym_order(int sym) { return sym == kSymNone ? 1 : sym == kSymQuarter ? 4 : 2; }
+
+// Up to four images that share lists, processed together: the images of one
+// instance, or of several instances of one geometry.
+struct WinGroup {
+    int64_t mbar_off[4];           // first weight of each image (the last repeated past n_img)
+    int64_t block0;                // the geometry's first block
+    int64_t det_off, ray_off;      // its fixed-point detectors and directions
+    int32_t tile0;                 // pixel sums of image c of patch p: tile tile0 + p * n_img + c
+    int32_t n_blocks, n_img;
+    int32_t zinfo_off;             // its patch records
+    int32_t flip;                  // bit c: image c's detectors run backwards from mbar_off
+    int32_t m_mask;                // m_pitch - 1
+    uint32_t ray_rec0, slot_rec0, code0;   // records and codes of its first block
+};
+
+// Share of one warp: `count` blocks from block `block` of group `group` on
+// (running into the following groups); its part of its first patch is the
+// patch's `part`-th.
+struct WinShare {
+    int32_t group, block, count, part;
+    uint32_t ray_rec, slot_rec, code, pad;   // records and codes of its first block
+};
+
 // Tile of the elementwise / stencil kernels: 32 x 8 pixels.
 struct ImgTile {
     int32_t inst, x0, y0, pad;
@@ -180,6 +263,18 @@ struct DevPlan {
     const uint32_t* codes;         // adjoint lists: the blocks (codes, or indices and fractions)
     const ListItem* list_items;    // adjoint list mode: (patch, part) items, grouped by warp
     const int32_t* warp_items;     // adjoint list mode: first item of each warp (+ end)
+    const uint4* win_heads;        // windowed lists: block heads, groups, warp shares, staging records, codes
+    const WinGroup* win_groups;
+    const WinShare* win_shares;    //   (groups of four instances, then of two, then single ones)
+    const uint2* win_rays;         //   per 4 staged rays: j | centre radius << 14, first ray | its slot << 16
+    const uint32_t* win_slots;     //   per 8 staged radii: index of the first in Mbar
+    const uint2* win_codes;        //   entry: ray byte offset | 4 x radius slot << 16
+    const int2* win_zinfo;         //   per (group, patch): first tile of its parts, parts
+    int32_t* win_arrived;          //   and the parts finished (zero between launches)
+    const int4* win_det;           // detector in 32.32 fixed point: fractions (u, v), integer parts (u, v)
+    const uint4* win_dirs;         // direction modulo one pixel, 0.64 fixed point: high words (u, v), low words (u, v)
+    const int2* win_dirs_int;      //   and its integer parts (list building)
+    float* win_z;                  // pixel-sum tiles: every group's sums, then the parts of split patches
     float* mpart;                  // forward partial slots
     float* msum;                   // forward circular-mean sums M (same layout as Mbar)
     int32_t* work_counters;        // dynamic work queues, kQueueStride ints apart (see kQueueStride)
@@ -203,6 +298,8 @@ struct DevPlan {
     int32_t bounds_probe;          // test hook (debug builds): the next list gather plants one
                                    //   out-of-range detector index for its bounds check to report
     int64_t n_code_vecs;           // adjoint lists: 16-byte vectors in the codes buffer
+    int64_t n_win_vecs;            // windowed lists: code vectors (256 bytes each); 0 = not in use
+    int32_t win_n_warps[3];        //   warps of the launches for groups of four, two and one
     int32_t list_tail0;            // adjoint lists: list_items[list_tail0 ..] is the shared tail queue
     int32_t n_tail_items;          //   of small items (largest first), after the per-warp items
     int32_t abel_cluster_fwd;      // CTAs per cluster splitting each forward time contraction

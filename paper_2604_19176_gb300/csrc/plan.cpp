@@ -201,6 +201,21 @@ void choose_tile(int n, int64_t cells, int want_w, int want_h, int& tw, int& th)
     }
 }
 
+// x as whole + frac / 2^64
+struct Fixed {
+    int32_t whole;
+    uint64_t frac;
+};
+Fixed fixed_of(double x)
+{
+    double w = std::floor(x), f = x - w;
+    if (f >= 1.0) {   // (x a rounding error below a whole number)
+        w += 1.0;
+        f = 0.0;
+    }
+    return {(int32_t)w, (uint64_t)(f * 18446744073709551616.0)};
+}
+
 } // namespace
 
 static_assert(sizeof(InstDev) % 8 == 0, "InstDev layout");
@@ -272,6 +287,12 @@ pat_status_t build_plan(Plan& P, const pat_geometry_t* geoms, int n_inst, const 
     std::vector<float> detU, detV;     // FP32 detector coordinates (host geometry)
     std::vector<float4> det4, rays;
     std::vector<float2> rtrig;
+    // windowed adjoint lists (windows.cu), the default where their staged
+    // tables hold a patch's radii: detectors and directions in fixed point
+    const bool win_wanted = opt.adj_mode == 0 && opt.adj_groups == 0 && opt.adj_jblock == 0 && windows_fit(geoms, n_inst);
+    std::vector<int4> win_det;
+    std::vector<uint4> win_dirs;
+    std::vector<int2> win_dirs_int;
     std::vector<InstDev> inst(n_inst);
     int64_t tile_bytes = 0;
     int tiles_max = 0;
@@ -320,6 +341,18 @@ pat_status_t build_plan(Plan& P, const pat_geometry_t* geoms, int n_inst, const 
             detV.push_back(vf);
             const double ui = std::floor((double)uf), vi = std::floor((double)vf);
             det4.push_back(make_float4((float)ui, (float)vi, (float)(ue - ui), (float)(ve - vi)));
+            if (win_wanted) {
+                const Fixed u = fixed_of(ue), v = fixed_of(ve);
+                // (32 fraction bits, rounded; a carry goes to the integer part)
+                auto hi32 = [](const Fixed& f, int32_t& whole) {
+                    const uint64_t r = (f.frac >> 32) + ((f.frac >> 31) & 1u);
+                    whole = f.whole + (int32_t)(r >> 32);
+                    return (int32_t)(uint32_t)r;
+                };
+                int32_t iu = 0, iv = 0;
+                const int32_t fu = hi32(u, iu), fv = hi32(v, iv);
+                win_det.push_back(make_int4(fu, fv, iu, iv));
+            }
         }
         // M / Mbar row pitch and the adjoint list code q << (jb + mb) | j << mb | m
         {
@@ -344,6 +377,16 @@ pat_status_t build_plan(Plan& P, const pat_geometry_t* geoms, int n_inst, const 
                 const float ch = (float)dc, sh = (float)ds;
                 rays.push_back(make_float4(ch, sh, (float)(dc - (double)ch), (float)(ds - (double)sh)));
                 rtrig.push_back(make_float2(rcp(ch), rcp(sh)));
+            }
+            if (win_wanted) {   // (a few entries past K: staged rays come in fours)
+                d.win_ray_off = (int64_t)win_dirs.size();
+                for (int q = 0; q < g.n_angles + 4; ++q) {
+                    const double ph = kTwoPi * (q % g.n_angles) / g.n_angles;
+                    const Fixed x = fixed_of(delta * std::cos(ph)), y = fixed_of(delta * std::sin(ph));
+                    win_dirs.push_back(make_uint4((uint32_t)(x.frac >> 32), (uint32_t)(y.frac >> 32), (uint32_t)x.frac,
+                                                  (uint32_t)y.frac));
+                    win_dirs_int.push_back(make_int2(x.whole, y.whole));
+                }
             }
         }
 
@@ -612,7 +655,10 @@ pat_status_t build_plan(Plan& P, const pat_geometry_t* geoms, int n_inst, const 
                     : (double)slot_samples_all * 12.0 <= budget                  ? 3
                                                                                  : 2;
     }
-    const bool use_lists = list_mode == 1 || list_mode == 3 || list_mode == 4;
+    // the windowed form of the code lists takes their place under the same
+    // budget (its codes are 4 B per entry too); its codes never run out of bits
+    const bool use_win = win_wanted && (double)slot_samples_all * 4.0 * 1.5 <= (double)P.list_budget_bytes;
+    const bool use_lists = !use_win && (list_mode == 1 || list_mode == 3 || list_mode == 4);
     const bool frac_lists = list_mode == 3;
     const int list_lm = list_mode == 3 ? 1 : list_mode == 4 ? 2 : 0;
     // detectors per aligned block of the code lists (measured best at 8 on
@@ -623,7 +669,7 @@ pat_status_t build_plan(Plan& P, const pat_geometry_t* geoms, int n_inst, const 
     // Items with an estimate of their cost (candidate rays per detector, from
     // the patch centre), sorted largest first for the kernel's dynamic queue.
     std::vector<std::pair<double, CellItem>> wit;
-    for (int i = 0; i < n_inst; ++i) {
+    for (int i = 0; i < (use_win || use_lists ? 0 : n_inst); ++i) {
         const InstDev& d = inst[i];
         const int n = geoms[i].n;
         const double R = 0.7111, per_rad = d.K / kTwoPi;
@@ -652,7 +698,7 @@ pat_status_t build_plan(Plan& P, const pat_geometry_t* geoms, int n_inst, const 
         LG = opt.adj_groups > 0 ? opt.adj_groups
                                 : (int)std::max<int64_t>(1, std::min<int64_t>(16, (2 * lres + patches - 1) / patches));
     }
-    const int ZG = use_lists ? LG : AG;
+    const int ZG = use_win ? 0 : use_lists ? LG : AG;
     std::vector<CellItem> citems;
     citems.reserve(wit.size());
     for (auto& w : wit) citems.push_back(w.second);
@@ -750,6 +796,9 @@ pat_status_t build_plan(Plan& P, const pat_geometry_t* geoms, int n_inst, const 
     const size_t o_det = reserve(sizeof(float4) * det4.size());
     const size_t o_rays = reserve(sizeof(float4) * rays.size());
     const size_t o_rtrig = reserve(sizeof(float2) * rtrig.size());
+    const size_t o_wdet = reserve(sizeof(int4) * win_det.size());
+    const size_t o_wdirs = reserve(sizeof(uint4) * win_dirs.size());
+    const size_t o_wdint = reserve(sizeof(int2) * win_dirs_int.size());
     const size_t o_P = reserve(sizeof(float) * pmat.size());
     const size_t o_slot = reserve(sizeof(int32_t) * slotcnt.size());
     const size_t o_units = reserve(sizeof(Unit) * units.size());
@@ -778,6 +827,9 @@ pat_status_t build_plan(Plan& P, const pat_geometry_t* geoms, int n_inst, const 
     put(o_det, det4.data(), sizeof(float4) * det4.size());
     put(o_rays, rays.data(), sizeof(float4) * rays.size());
     put(o_rtrig, rtrig.data(), sizeof(float2) * rtrig.size());
+    put(o_wdet, win_det.data(), sizeof(int4) * win_det.size());
+    put(o_wdirs, win_dirs.data(), sizeof(uint4) * win_dirs.size());
+    put(o_wdint, win_dirs_int.data(), sizeof(int2) * win_dirs_int.size());
     put(o_P, pmat.data(), sizeof(float) * pmat.size());
     put(o_slot, slotcnt.data(), sizeof(int32_t) * slotcnt.size());
     put(o_units, units.data(), sizeof(Unit) * units.size());
@@ -796,7 +848,7 @@ pat_status_t build_plan(Plan& P, const pat_geometry_t* geoms, int n_inst, const 
     // workspace (floats): forward slots | Mbar | TV partials | (aligned) cell sums (float4)
     // workspace (4-byte words): slots | M | Mbar | TV partials | arrival counters | cell sums (float4)
     const int64_t tv_parts = 3 * (int64_t)itiles.size();
-    const int64_t o_msum = mpart_total, o_mbar = o_msum + mbar_total, o_tvp = o_mbar + mbar_total;
+    const int64_t o_msum = (mpart_total + 63) / 64 * 64, o_mbar = o_msum + mbar_total, o_tvp = o_mbar + mbar_total;
     const int64_t o_ctr = ((o_tvp + tv_parts + kQueueStride - 1) / kQueueStride) * kQueueStride;
     const int64_t n_ctr = 2 * (int64_t)kQueueStride;
     const int64_t o_res = ((o_ctr + n_ctr + 63) / 64) * 64;   // data residual of pat_tv_step
@@ -820,6 +872,9 @@ pat_status_t build_plan(Plan& P, const pat_geometry_t* geoms, int n_inst, const 
     dp.det = reinterpret_cast<const float4*>(base + o_det);
     dp.rays = reinterpret_cast<const float4*>(base + o_rays);
     dp.rtrig = reinterpret_cast<const float2*>(base + o_rtrig);
+    dp.win_det = reinterpret_cast<const int4*>(base + o_wdet);
+    dp.win_dirs = reinterpret_cast<const uint4*>(base + o_wdirs);
+    dp.win_dirs_int = reinterpret_cast<const int2*>(base + o_wdint);
     dp.P = reinterpret_cast<const float*>(base + o_P);
     dp.slotcnt = reinterpret_cast<const uint8_t*>(base + o_slot);
     dp.units = reinterpret_cast<const Unit*>(base + o_units);
@@ -896,6 +951,13 @@ pat_status_t build_plan(Plan& P, const pat_geometry_t* geoms, int n_inst, const 
     // count of the patch's cells sets the block's segment; the segments make
     // the patch's sequence, cut into G equal parts (fill in k_adj_seg).
     int64_t list_bytes = 0;
+    if (use_win) {
+        int parts = 1;
+        const pat_status_t s = build_windows(P, inst, inst_tmpl, (int)tmpls.size(),
+                                             reinterpret_cast<InstDev*>(base + o_inst), &list_bytes, &parts, st);
+        if (s != PAT_OK) return s;
+        dp.adj_groups = parts;
+    }
     if (use_lists) {
         const int S = frac_lists ? 3 : 1;     // 16-byte slots per vector of four entries
         const int G = LG;
@@ -1210,7 +1272,8 @@ pat_status_t build_plan(Plan& P, const pat_geometry_t* geoms, int n_inst, const 
             I.tile_cols = std::max(I.tile_cols, t.x1 - t.x0);
         }
     I.adj_groups = dp.adj_groups;
-    I.adj_mode = dp.adj_mode == 0 ? 2 : dp.adj_mode;
+    I.adj_mode = use_win ? (pairs_fit ? 4 : 1) : dp.adj_mode == 0 ? 2 : dp.adj_mode;
+    I.adj_windows = use_win ? 1 : 0;
     I.abel_split_fwd = dp.abel_cluster_fwd;
     I.abel_split_adj = dp.abel_cluster_adj;
     I.time_pair = dp.time_chunks > 0 ? 1 : 0;
@@ -1252,7 +1315,9 @@ void free_plan_memory(Plan& P)
     if (P.d_tables) cudaFree(P.d_tables);
     if (P.d_work) cudaFree(P.d_work);
     if (P.d_lists) cudaFree(P.d_lists);
+    if (P.d_codes) cudaFree(P.d_codes);
     P.d_lists = nullptr;
+    P.d_codes = nullptr;
     P.d_tables = nullptr;
     P.d_work = nullptr;
 }

@@ -29,7 +29,8 @@ struct Plan {
     int64_t work_floats = 0;
     int32_t* d_counters = nullptr;     // arrival counters + work queues (zero between calls)
     size_t counters_bytes = 0;
-    void* d_lists = nullptr;           // adjoint sample lists (list mode)
+    void* d_lists = nullptr;           // adjoint sample lists (list mode); blocks and records (windowed lists)
+    void* d_codes = nullptr;           // windowed lists: codes, warp shares, pixel sums
     float* d_resid = nullptr;          // data residual of the fused TV step (inside d_work)
     int code_bits_max = 0;             // bits of a packed (j, m, q) sample code, largest instance
     int64_t list_budget_bytes = 24ll << 30;
@@ -47,6 +48,15 @@ struct Plan {
 pat_status_t build_plan(Plan& P, const pat_geometry_t* geoms, int n_inst, const pat_options_t& opt,
                         cudaStream_t st);
 void free_plan_memory(Plan& P);
+
+// Windowed adjoint lists (windows_plan.cpp).  windows_fit: whether the staged
+// tables hold every geometry's windows.  build_windows builds them for the
+// plan's instances (inst_tmpl: the geometry template of each) on `st`, fills
+// dp.win_* and the instances' fields (uploaded to d_inst), and gives the
+// device bytes and the most parts a patch is split into.
+bool windows_fit(const pat_geometry_t* geoms, int n_inst);
+pat_status_t build_windows(Plan& P, std::vector<InstDev>& inst, const std::vector<int>& inst_tmpl, int n_tmpl,
+                           InstDev* d_inst, int64_t* bytes, int* parts_max, cudaStream_t st);
 
 // Every device allocation of plan creation (and of the autotuner) goes
 // through dev_malloc.  Test hook: after set_alloc_failure(n), the n-th next
