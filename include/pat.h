@@ -105,9 +105,10 @@ typedef struct {
     int32_t band_rows;   /* max pixel rows of a circular-mean tile; 0 = auto                 */
     int32_t adj_groups;  /* detector groups of the adjoint gather, 1..16; 0 = auto           */
     int32_t adj_mode;    /* adjoint gather: 0 = auto (windowed code lists where adj_groups    */
-                         /*   and adj_jblock are 0 too, a 16-pixel patch's radii fit the      */
+                         /*   and adj_jblock are 0 too, the radii that cross 8 pixels fit the */
                          /*   staged tables and the codes the list budget; else 4 if it fits  */
-                         /*   the budget, else 1, else 3, else 2); 1 = per-cell sample code lists built at        */
+                         /*   the budget, else 1, else 3, else 2);                            */
+                         /*   1 = per-cell sample code lists built at                         */
                          /*   creation (device memory ~4 B per sample); 2 = enumerate on      */
                          /*   every call (no list memory); 3 = per-cell fraction lists built  */
                          /*   at creation (~12 B per sample: Mbar index and the FP32 bilinear */

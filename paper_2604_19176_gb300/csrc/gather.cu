@@ -14,14 +14,16 @@
 // that can land in it, and each candidate's cell is re-evaluated with exactly
 // the forward's split-form expression.  Hits come out in the order (j, q, m).
 //
-// Three ways to run this:
+// The default gather, over windowed lists, is in windows.cu; the forms here
+// serve the options that ask for them and the geometries that its staged
+// tables do not hold.  Three ways to run this:
 //   code lists (when 4 B per sample fits the list budget and a (q, j, m)
 //     code fits 32 bits): at plan creation the enumeration runs twice
 //     (count, then fill) to store every cell's hits as packed codes, the 32
 //     cells of an 8 x 4 patch interleaved vector by vector so that a warp
 //     streams them with full 512-byte loads; each call recomputes a and b
 //     from the codes with the forward's expressions (k_adj_list).  The
-//     default form is run pairs: most hits of a cell come in runs of two
+//     shorter form is run pairs: most hits of a cell come in runs of two
 //     consecutive radii on one ray (a cell is about two radius steps wide),
 //     and one code then stands for both, so the pair shares its detector and
 //     ray loads and the code stream shrinks by about 40 %.

@@ -49,6 +49,16 @@
 // Instances with the same geometry share lists in the same way.  Up to four
 // images are processed together (NB): the code, the staged ray and the
 // fractions serve all, and their weights sit side by side in shared memory.
+//
+// Bound by the L1 data path, which shared memory shares: about 10 wavefronts
+// per 32 real samples for one image, most of them the 16-byte ray of every
+// entry, 6 for two images and 4.5 for four; issue slots are half used.  At
+// 512^2 (256 detectors on a half ring, pairs of images) ncu counts 27 M shared
+// wavefronts and 79 M warp instructions, 70 % of the L1 data path's peak.
+// Gather and combine, per-cell run-pair lists -> windowed lists: 49 -> 32 us
+// at 256^2 (128 detectors, half ring), 328 -> 139 us at 512^2, 595 -> 330 us
+// at 760^2 (256 detectors, 270 degrees), 3.53 -> 1.98 ms for 64 uneven
+// instances, 13.4 -> 5.3 ms for 8 x 1024^2.
 #include <algorithm>
 
 #include "device_common.cuh"
@@ -151,6 +161,8 @@ __device__ __forceinline__ float lds32(uint32_t addr)
     return v;
 }
 
+// 20 warps per SM (96 registers; 16 for four images): 24 warps at 80 registers
+// took 150 instead of 144 us at 512^2, and left L1 too little room.
 template <int NB>
 __global__ void __launch_bounds__(kWinThreads, NB == 4 ? 4 : 5) k_adj_win(DevPlan dp, int warp0, int n_warps)
 {
