@@ -8,24 +8,26 @@
 // lower triangular plus one super-diagonal, so a tile of outputs only needs
 // the band of the contraction where its slice of P is nonzero.
 //
-// Both stages are C[j][x] = sum_k A[j][k] B[k][x] over a 32 x 32 output tile
-// (32 detectors, 32 times or radii): A = M and B = P^T for the forward,
-// A = gbar and B = P for the adjoint.  Warp w owns detectors 4w .. 4w+3 and
-// lane l output x0 + l, so each thread keeps four FP32 accumulators and each
-// staged element of P serves 32 detectors.  Every output is a sequential
-// FMA chain over k in increasing order.
+// Both stages are C[j][x] = sum_k A[j][k] B[k][x] over a T x T output tile
+// (T detectors, T times or radii): A = M and B = P^T for the forward,
+// A = gbar and B = P for the adjoint.  With T = 64 each of 128 threads owns 8
+// detectors x 4 outputs: a step of k costs it three 16-byte shared-memory reads
+// for 32 FMAs.  With T = 32 each of 256 threads owns 2 x 2 (two reads for four
+// FMAs), for plans too small to fill the SMs with 64 x 64 tiles.
 //
 // The contraction runs in chunks of 32 rows through a ring of kStages
-// shared-memory stages filled by asynchronous copies (16-byte copies for the
-// chunk of P, 4-byte zero-filling copies that write the chunk of A already
-// transposed, so that a warp reads its four detectors as one broadcast
-// 16-byte load), kStages - 1 chunks ahead of the FMAs: a CTA's loads are all
-// in flight at once for short contractions.
+// shared-memory stages filled by asynchronous copies: 16-byte copies for the
+// chunk of B, 4-byte zero-filling copies that write the chunk of A already
+// transposed (8 rows x 4 detectors per warp, so that each fetches whole
+// 32-byte sectors and no two of its lanes write the same bank).
 //
-// When a plan has fewer tiles than SMs, a thread-block cluster of 2, 4 or 8 CTAs
-// shares each tile: rank r takes the r-th share of the chunks, and rank 0
-// adds the partial tiles in rank order through distributed shared memory
-// (deterministic; no global atomics).
+// A thread-block cluster of 2, 4 or 8 CTAs shares each tile where there are
+// too few tiles for the SMs: rank r takes the r-th share of the chunks, and
+// every rank adds its share of the tile's rows over all partial tiles in rank
+// order through distributed shared memory (deterministic; no global atomics).
+//
+// Bound by the FMA pipe on large plans, by the latency of its few chunks, the
+// cluster barriers and the launch on small ones.
 #include <cooperative_groups.h>
 
 #include "device_common.cuh"
@@ -35,15 +37,39 @@ namespace patgpu {
 
 namespace cg = cooperative_groups;
 
-static_assert(kAbelJ == 4 * kAbelWarps && kAbelX == kWarp && kAbelKC == 32, "Abel tile shape");
+static_assert(kAbelKC == 32, "Abel tile shape");
 
 namespace {
-constexpr int kStages = 6;
+template <int T>
 struct AbelSmem {
-    float A[kStages][kAbelKC][kAbelJ + 4];   // [stage][k][detector], rows 16-byte aligned
-    float B[kStages][kAbelKC][kAbelX];       // [stage][k][output]
-    float part[kAbelJ][kAbelX];              // partial tile read by cluster rank 0
+    static constexpr int kStages = T == 64 ? 3 : 6;
+    static constexpr int kWarps = T == 64 ? 4 : 8;
+    float A[kStages][kAbelKC][T + 4];   // [stage][k][detector], rows 16-byte aligned
+    float B[kStages][kAbelKC][T];       // [stage][k][output]
+    // after the contraction: the partial tile [detector][output], read by the other ranks
 };
+static_assert(sizeof(AbelSmem<64>) >= sizeof(float) * 64 * 64 && sizeof(AbelSmem<32>) >= sizeof(float) * 32 * 32,
+              "partial tile");
+
+// N consecutive values from shared memory
+template <int N>
+__device__ __forceinline__ void lds_vec(const float* p, float (&v)[N])
+{
+    if constexpr (N % 4 == 0) {
+#pragma unroll
+        for (int i = 0; i < N; i += 4) {
+            const float4 t = *reinterpret_cast<const float4*>(p + i);
+            v[i] = t.x;
+            v[i + 1] = t.y;
+            v[i + 2] = t.z;
+            v[i + 3] = t.w;
+        }
+    } else {
+        const float2 t = *reinterpret_cast<const float2*>(p);
+        v[0] = t.x;
+        v[1] = t.y;
+    }
+}
 } // namespace
 
 // FWD: gin unused, gout = g (gsub nullable: gout = A f - gsub).
@@ -52,14 +78,17 @@ struct AbelSmem {
 //   primal-dual iteration (the proximal map of the conjugate of
 //   1/2 ||. - g||^2), with inv1ps = 1 / (1 + sigma).
 // ADJ: gin = gbar, gout unused (writes Mbar in the plan workspace).
-template <bool FWD, bool DUAL>
-__global__ void __launch_bounds__(kAbelWarps * kWarp) k_abel(DevPlan dp, const float* __restrict__ gin,
+template <int T, bool FWD, bool DUAL>
+__global__ void __launch_bounds__(AbelSmem<T>::kWarps * kWarp) k_abel(DevPlan dp, const float* __restrict__ gin,
                                                              float* __restrict__ gout,
                                                              const float* __restrict__ gsub, int cs, float sigma,
                                                              float inv1ps)
 {
     extern __shared__ __align__(16) unsigned char abel_smem[];
-    AbelSmem& sm = *reinterpret_cast<AbelSmem*>(abel_smem);
+    using Smem = AbelSmem<T>;
+    constexpr int kStages = Smem::kStages, NW = Smem::kWarps, NT = NW * kWarp;
+    constexpr int MX = T / 16, MJ = T * T / NT / MX;   // a thread owns MJ detectors x MX outputs
+    Smem& sm = *reinterpret_cast<Smem*>(abel_smem);
     const int rank = (int)(blockIdx.x % (unsigned)cs);
     const TimeTile t = (FWD ? dp.fwd_tiles : dp.adj_tiles)[blockIdx.x / cs];
     const InstDev in = dp.inst[t.inst];
@@ -75,7 +104,7 @@ __global__ void __launch_bounds__(kAbelWarps * kWarp) k_abel(DevPlan dp, const f
         B = dp.P + in.p_off + (size_t)in.n_tp * in.n_rp;
         b_pitch = in.n_tp;
         k_begin = 0;
-        k_end = min(in.n_r, t.x0 + kAbelX + 2);
+        k_end = min(in.n_r, t.x0 + T + 2);
     } else {
         A = gin + in.g_off;
         a_pitch = in.n_t;
@@ -89,110 +118,127 @@ __global__ void __launch_bounds__(kAbelWarps * kWarp) k_abel(DevPlan dp, const f
     const int per = (nchunks + cs - 1) / cs;
     const int c_lo = min(nchunks, rank * per), c_hi = min(nchunks, c_lo + per);
 
-    // copy roles: A elements (detector ja, rows ka .. ka+3); B (row rb, columns cb .. cb+3)
-    const int ja = tid >> 3, ka = (tid & 7) * 4;
-    const int rb = tid >> 3, cb = (tid & 7) * 4;
-    const bool ja_ok = t.j0 + ja < in.n_det;
-    const float* Arow = A + (size_t)(ja_ok ? t.j0 + ja : 0) * a_pitch;
-    // issues chunk c into its stage; always commits one group (empty past the end)
-    auto issue = [&](int c) {
-        if (c < c_hi) {
-            const int st = (c - c_lo) % kStages;
-            const int k0 = k_begin + c * kAbelKC;
-            cp_async16(&sm.B[st][rb][cb], B + (size_t)(k0 + rb) * b_pitch + t.x0 + cb);
+    // copy roles of a warp: B rows, 16 bytes per lane; A elements (8 k x 4 detectors per copy)
+    auto issue_b = [&](int c) {
+        if (c >= c_hi) return;
+        const int st = (c - c_lo) % kStages, k0 = k_begin + c * kAbelKC;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int k = k0 + ka + i;
-                const bool ok = ja_ok && k < a_len;
-                cp_async4_zfill(&sm.A[st][ka + i][ja], ok ? Arow + k : Arow, ok);
-            }
+        for (int i = 0; i < T * 8 / NT; ++i) {
+            const int row = tid / (T / 4) + NT / (T / 4) * i, col = tid % (T / 4) * 4;
+            const bool ok = t.x0 + col < b_pitch;   // (the pitch is a multiple of 32)
+            cp_async16_zfill(&sm.B[st][row][col], B + (size_t)(k0 + row) * b_pitch + (ok ? t.x0 + col : 0), ok);
         }
-        cp_async_commit();
+    };
+    auto issue_a = [&](int c) {
+        if (c >= c_hi) return;
+        const int st = (c - c_lo) % kStages, k0 = k_begin + c * kAbelKC;
+        const int kl = (lane & 7) + 8 * (w & 3), jl = (lane >> 3) + T * 4 / NW * (w >> 2);
+        const int k = k0 + kl;
+        const bool k_ok = k < a_len;
+        const float* src = A + (size_t)(t.j0 + jl) * a_pitch + k;
+#pragma unroll
+        for (int i = 0; i < T / NW; ++i) {
+            const bool ok = k_ok && t.j0 + jl + 4 * i < in.n_det;
+            cp_async4_zfill(&sm.A[st][kl][jl + 4 * i], ok ? src + (size_t)(4 * i) * a_pitch : A, ok);
+        }
     };
 
-    pdl_wait();   // M (forward) or gbar (adjoint) come from the previous kernel
-    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    // P does not depend on the data: its first chunks before the dependency wait
 #pragma unroll
-    for (int i = 0; i < kStages - 1; ++i) issue(c_lo + i);
+    for (int i = 0; i < kStages - 1; ++i) issue_b(c_lo + i);
+    pdl_wait();   // M (forward) or gbar (adjoint) come from the previous kernel
+#pragma unroll
+    for (int i = 0; i < kStages - 1; ++i) {
+        issue_a(c_lo + i);
+        cp_async_commit();   // (the first group holds every early chunk of B)
+    }
+    const int tx = tid & 15, ty = tid >> 4;   // outputs MX tx .., detectors MJ ty ..
+    float acc[MJ][MX];
+#pragma unroll
+    for (int i = 0; i < MJ; ++i)
+#pragma unroll
+        for (int j = 0; j < MX; ++j) acc[i][j] = 0.f;
     for (int c = c_lo; c < c_hi; ++c) {
         const int st = (c - c_lo) % kStages;
         cp_async_wait_group<kStages - 2>();   // chunk c has landed (this thread's copies)
-        __syncthreads();                      // ... and every thread's
+        __syncthreads();                      // ... and every thread's; the stage of chunk c - 1 is free
+        issue_b(c + kStages - 1);
+        issue_a(c + kStages - 1);
+        cp_async_commit();
 #pragma unroll 8
         for (int k = 0; k < kAbelKC; ++k) {
-            const float b = sm.B[st][k][lane];
-            const float4 a = *reinterpret_cast<const float4*>(&sm.A[st][k][4 * w]);
-            acc.x = fmaf(b, a.x, acc.x);
-            acc.y = fmaf(b, a.y, acc.y);
-            acc.z = fmaf(b, a.z, acc.z);
-            acc.w = fmaf(b, a.w, acc.w);
+            float av[MJ], bv[MX];
+            lds_vec<MJ>(&sm.A[st][k][MJ * ty], av);
+            lds_vec<MX>(&sm.B[st][k][MX * tx], bv);
+#pragma unroll
+            for (int i = 0; i < MJ; ++i)
+#pragma unroll
+                for (int j = 0; j < MX; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
         }
-        __syncthreads();                      // stage st is free again
-        issue(c + kStages - 1);
     }
     cp_async_wait_group<0>();
 
-    if (cs > 1) {
-        cg::cluster_group cluster = cg::this_cluster();
-        sm.part[4 * w + 0][lane] = acc.x;
-        sm.part[4 * w + 1][lane] = acc.y;
-        sm.part[4 * w + 2][lane] = acc.z;
-        sm.part[4 * w + 3][lane] = acc.w;
-        cluster.sync();
-        if (rank == 0) {
-            float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-            for (int r = 0; r < cs; ++r) {
-                const float* pr = cluster.map_shared_rank(&sm.part[0][0], r);
-                s.x += pr[(4 * w + 0) * kAbelX + lane];
-                s.y += pr[(4 * w + 1) * kAbelX + lane];
-                s.z += pr[(4 * w + 2) * kAbelX + lane];
-                s.w += pr[(4 * w + 3) * kAbelX + lane];
-            }
-            acc = s;
+    auto store = [&](int j, int x, float v) {   // detector and output of the instance
+        if (FWD) {
+            if (j >= in.n_det || x >= in.n_t) return;
+            const size_t o = in.g_off + (size_t)j * in.n_t + x;
+            v *= in.inv_K;
+            if (DUAL)
+                gout[o] = fmaf(sigma, v - gsub[o], gout[o]) * inv1ps;
+            else
+                gout[o] = gsub ? v - gsub[o] : v;
+        } else {
+            if (j >= in.n_det || x >= in.n_r) return;
+            dp.mbar[in.mbar_off + (size_t)j * in.m_pitch + x] = v;
         }
-        cluster.sync();   // keep every rank's partial alive until rank 0 has read it
-        if (rank != 0) return;
-    }
-
-    const float r4[4] = {acc.x, acc.y, acc.z, acc.w};
-    const int x = t.x0 + lane;
-    if (FWD) {
-        if (x < in.n_t) {
+    };
+    if (cs == 1) {
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int j = t.j0 + 4 * w + i;
-                if (j >= in.n_det) break;
-                const size_t o = in.g_off + (size_t)j * in.n_t + x;
-                const float v = r4[i] * in.inv_K;
-                if (DUAL)
-                    gout[o] = fmaf(sigma, v - gsub[o], gout[o]) * inv1ps;
-                else
-                    gout[o] = gsub ? v - gsub[o] : v;
-            }
-        }
-    } else {
-        if (x < in.n_r) {
+        for (int i = 0; i < MJ; ++i)
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int j = t.j0 + 4 * w + i;
-                if (j >= in.n_det) break;
-                dp.mbar[in.mbar_off + (size_t)j * in.m_pitch + x] = r4[i];
-            }
-        }
+            for (int j = 0; j < MX; ++j) store(t.j0 + MJ * ty + i, t.x0 + MX * tx + j, acc[i][j]);
+        return;
     }
+    cg::cluster_group cluster = cg::this_cluster();
+    float* part = reinterpret_cast<float*>(abel_smem);
+    __syncthreads();   // every warp is done with the staged chunks
+#pragma unroll
+    for (int i = 0; i < MJ; ++i)
+#pragma unroll
+        for (int j = 0; j < MX; ++j) part[(MJ * ty + i) * T + MX * tx + j] = acc[i][j];
+    cluster.sync();
+    const int rows = T / cs;
+    for (int e = tid; e < rows * T; e += NT) {
+        const int j = rank * rows + e / T, x = e % T;
+        float v[8];
+#pragma unroll
+        for (int r = 0; r < 8; ++r) v[r] = r < cs ? cluster.map_shared_rank(part, r)[j * T + x] : 0.f;
+        float s = 0.f;
+#pragma unroll
+        for (int r = 0; r < 8; ++r) s += v[r];
+        store(t.j0 + j, t.x0 + x, s);
+    }
+    cluster.sync();   // every rank's partial stays until all have read it
 }
 
 namespace {
+template <int T, bool FWD, bool DUAL>
+cudaError_t launch_abel_t(const DevPlan& dp, int tiles, int cs, const float* gin, float* gout, const float* gsub,
+                          cudaStream_t st, float sigma, float inv1ps)
+{
+    cudaError_t e = cudaFuncSetAttribute(k_abel<T, FWD, DUAL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)sizeof(AbelSmem<T>));
+    if (e != cudaSuccess) return e;
+    return launch_pdl(k_abel<T, FWD, DUAL>, dim3((unsigned)(tiles * cs)),
+                      dim3(AbelSmem<T>::kWarps * kWarp), sizeof(AbelSmem<T>), st, cs, dp, gin, gout, gsub, cs, sigma, inv1ps);
+}
 template <bool FWD, bool DUAL = false>
 cudaError_t launch_abel(const DevPlan& dp, int tiles, int cs, const float* gin, float* gout, const float* gsub,
                         cudaStream_t st, float sigma = 0.f, float inv1ps = 1.f)
 {
     if (tiles == 0) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(k_abel<FWD, DUAL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)sizeof(AbelSmem));
-    if (e != cudaSuccess) return e;
-    return launch_pdl(k_abel<FWD, DUAL>, dim3((unsigned)(tiles * cs)), dim3(kAbelWarps * kWarp), sizeof(AbelSmem),
-                      st, cs, dp, gin, gout, gsub, cs, sigma, inv1ps);
+    return dp.abel_tile == 64 ? launch_abel_t<64, FWD, DUAL>(dp, tiles, cs, gin, gout, gsub, st, sigma, inv1ps)
+                              : launch_abel_t<32, FWD, DUAL>(dp, tiles, cs, gin, gout, gsub, st, sigma, inv1ps);
 }
 } // namespace
 

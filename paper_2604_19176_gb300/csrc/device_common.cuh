@@ -301,6 +301,12 @@ __device__ __forceinline__ void cp_async4_zfill(void* dst, const void* src, bool
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(valid ? 4 : 0)
                  : "memory");
 }
+// 16-byte asynchronous copy that writes zeros when !valid (nothing is read then).
+__device__ __forceinline__ void cp_async16_zfill(void* dst, const void* src, bool valid)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(valid ? 16 : 0)
+                 : "memory");
+}
 __device__ __forceinline__ void cp_async_commit()
 {
     asm volatile("cp.async.commit_group;" ::: "memory");

@@ -98,8 +98,8 @@ struct Segment {
     int32_t pad[5];
 };
 
-// Output tile of the two Abel (time) stages: detectors [j0, j0 + kAbelJ),
-// outputs [x0, x0 + kAbelX) (times for the forward, radii for the adjoint).
+// Output tile of the two Abel (time) stages: detectors [j0, j0 + T), outputs
+// [x0, x0 + T) (times for the forward, radii for the adjoint), T = abel_tile.
 struct TimeTile {
     int32_t inst, j0, x0, pad;
 };
@@ -302,6 +302,7 @@ struct DevPlan {
     int32_t win_n_warps[3];        //   warps of the launches for groups of four, two and one
     int32_t list_tail0;            // adjoint lists: list_items[list_tail0 ..] is the shared tail queue
     int32_t n_tail_items;          //   of small items (largest first), after the per-warp items
+    int32_t abel_tile;             // side of the Abel tiles, 64 or 32
     int32_t abel_cluster_fwd;      // CTAs per cluster splitting each forward time contraction
     int32_t abel_cluster_adj;      // the same for the adjoint time contraction
     int32_t bf16;                  // image storage is BF16
@@ -312,9 +313,6 @@ struct DevPlan {
     int32_t time_smem_bytes;       // dynamic shared memory of the fused time stage
 };
 
-constexpr int kAbelJ = 32;         // detectors per Abel tile (4 per warp)
-constexpr int kAbelX = 32;         // outputs per Abel tile (one per lane)
-constexpr int kAbelWarps = 8;      // warps per Abel CTA
 constexpr int kAbelKC = 32;        // contraction rows staged per pipeline stage
 
 // Staged cells per row of a circular-mean tile `w` pixels wide: w + 3 cells,

@@ -159,6 +159,15 @@ struct GeomTemplate {
 };
 
 constexpr double kUnitOverhead = 24.0; // per-unit fixed cost, in angle iterations
+// Abel tiles of 64 from this many on (forward / adjoint time stage with tiles of
+// 32 and of 64: 10.8 / 10.9 and 12.7 / 11.8 us at 256^2, 128 detectors, 16
+// tiles of 64; 26.7 / 27.0 and 22 / 21 us at 512^2, 256 detectors, 64 tiles)
+constexpr int64_t kAbelTiles64 = 32;
+// The solver steps fuse the time stages up to this many multiply-adds: the one
+// launch saves two, but its 4-detector groups read P once per group (TV step
+// fused / separate: 67.7 / 72.7 us at 256^2 with 17 M; 138.9 / 114.7 us for
+// 16 x 128^2 with 34 M; 886 / 825 us at 760^2 with 529 M)
+constexpr int64_t kPairMacs = 24 << 20;
 constexpr double kListTailShare = 0.25; // list gather: share of the work in the shared tail queue
 
 // n pixels split into parts of at most w pixels, as equal as possible.
@@ -730,14 +739,19 @@ pat_status_t build_plan(Plan& P, const pat_geometry_t* geoms, int n_inst, const 
     }
 
     // ---- tiles --------------------------------------------------------------
+    // Abel tiles of 64 where there are enough of them that clusters of 8 can
+    // fill the SMs, else of 32
     std::vector<TimeTile> fwd_tiles, adj_tiles;
+    int64_t tiles64 = 0;
+    for (const InstDev& d : inst) tiles64 += (int64_t)((d.n_det + 63) / 64) * ((d.n_t + 63) / 64);
+    const int abel_tile = tiles64 >= kAbelTiles64 ? 64 : 32;
     std::vector<ImgTile> itiles;
     int64_t time_macs = 0;
     for (int i = 0; i < n_inst; ++i) {
         InstDev& d = inst[i];
-        for (int j0 = 0; j0 < d.n_det; j0 += kAbelJ) {
-            for (int k0 = 0; k0 < d.n_t; k0 += kAbelX) fwd_tiles.push_back({i, j0, k0, 0});
-            for (int m0 = 0; m0 < d.n_r; m0 += kAbelX) adj_tiles.push_back({i, j0, m0, 0});
+        for (int j0 = 0; j0 < d.n_det; j0 += abel_tile) {
+            for (int k0 = 0; k0 < d.n_t; k0 += abel_tile) fwd_tiles.push_back({i, j0, k0, 0});
+            for (int m0 = 0; m0 < d.n_r; m0 += abel_tile) adj_tiles.push_back({i, j0, m0, 0});
         }
         d.tile_off = (int32_t)itiles.size();
         for (int y0 = 0; y0 < d.n; y0 += 8)
@@ -749,7 +763,7 @@ pat_status_t build_plan(Plan& P, const pat_geometry_t* geoms, int n_inst, const 
     }
     // longest contractions first (the triangle makes late forward tiles and
     // early adjoint tiles heavier)
-    auto fwd_len = [&](const TimeTile& t) { return std::min(inst[t.inst].n_r, t.x0 + kAbelX + 2); };
+    auto fwd_len = [&](const TimeTile& t) { return std::min(inst[t.inst].n_r, t.x0 + abel_tile + 2); };
     auto adj_len = [&](const TimeTile& t) { return inst[t.inst].n_t - std::max(0, t.x0 - 2); };
     std::stable_sort(fwd_tiles.begin(), fwd_tiles.end(),
                      [&](const TimeTile& a, const TimeTile& b) { return fwd_len(a) > fwd_len(b); });
@@ -769,7 +783,7 @@ pat_status_t build_plan(Plan& P, const pat_geometry_t* geoms, int n_inst, const 
     std::stable_sort(tgroups.begin(), tgroups.end(),
                      [&](const TimeGroup& a, const TimeGroup& b) { return inst[a.inst].n_t > inst[b.inst].n_t; });
     int time_chunks = 0, time_smem = 0;
-    if (opt.time_pair == 0) {
+    if (opt.time_pair == 0 && time_macs <= kPairMacs) {
         const int chunks = (time_rows_r / 32 + kTimeCS - 1) / kTimeCS;   // n_rc >= n_tc
         const int64_t bytes = (int64_t)(time_rows_r + time_rows_t) * kTimeJ * 4 +
                               (int64_t)chunks * (kTimeWarps + 2) * kTimeJ * kWarp * 4;
@@ -778,10 +792,13 @@ pat_status_t build_plan(Plan& P, const pat_geometry_t* geoms, int n_inst, const 
             time_smem = (int)bytes;
         }
     }
-    // with fewer tiles than SMs, a cluster of CTAs splits each contraction
+    // with few tiles, a cluster of CTAs splits each contraction: up to 3.5 CTAs
+    // per SM of the 64 x 64 tiles, 2 of the smaller ones
     auto cluster_for = [&](size_t tiles) {
         if (opt.abel_split > 0) return (int)opt.abel_split;
-        return tiles >= (size_t)P.num_sms ? 1 : tiles * 2 >= (size_t)P.num_sms ? 2 : 4;
+        int cs = 8;
+        while (cs > 1 && 2 * tiles * cs > (size_t)P.num_sms * (abel_tile == 64 ? 7 : 4)) cs /= 2;
+        return cs;
     };
 
     // ---- upload -----------------------------------------------------------
@@ -916,6 +933,7 @@ pat_status_t build_plan(Plan& P, const pat_geometry_t* geoms, int n_inst, const 
     dp.cell_blocks = cell_blocks;
     dp.fwd_smem_bytes = smem_bytes;
     dp.fwd_rays_off = (int32_t)tile_bytes;
+    dp.abel_tile = abel_tile;
     dp.abel_cluster_fwd = cluster_for(fwd_tiles.size());
     dp.abel_cluster_adj = cluster_for(adj_tiles.size());
     dp.bf16 = bf16 ? 1 : 0;
