@@ -162,10 +162,8 @@ pat_status_t pat_plan_create(const pat_geometry_t* geoms, int32_t n_instances, c
     if (opt.schedule != PAT_SCHED_STAGED && opt.schedule != PAT_SCHED_PERSISTENT) return PAT_ERR_INVALID_ARG;
     if (opt.schedule == PAT_SCHED_PERSISTENT) return PAT_ERR_UNSUPPORTED;
     if (opt.tune < 0 || opt.tune > 2) return PAT_ERR_INVALID_ARG;
-    if (opt.m_lanes == 0) opt.m_lanes = 32;
-    if (opt.m_lanes != 32 && opt.m_lanes != 16 && opt.m_lanes != 8) return PAT_ERR_INVALID_ARG;
-    if (opt.q_piece == 0) opt.q_piece = 128;
-    if (opt.q_piece < 4 || opt.q_piece % 4 != 0) return PAT_ERR_INVALID_ARG;
+    if (opt.m_lanes != 0 && opt.m_lanes != 32 && opt.m_lanes != 16 && opt.m_lanes != 8) return PAT_ERR_INVALID_ARG;
+    if (opt.q_piece != 0 && (opt.q_piece < 4 || opt.q_piece % 4 != 0)) return PAT_ERR_INVALID_ARG;
     if (opt.band_rows != 0 && (opt.band_rows < 1 || opt.band_rows > 8192)) return PAT_ERR_INVALID_ARG;
     if (opt.tile_cols != 0 && (opt.tile_cols < 1 || opt.tile_cols > 8192)) return PAT_ERR_INVALID_ARG;
     if (opt.adj_groups < 0 || opt.adj_groups > 16) return PAT_ERR_INVALID_ARG;

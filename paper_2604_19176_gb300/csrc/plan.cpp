@@ -158,7 +158,9 @@ struct GeomTemplate {
     int64_t slot_samples = 0;        // lane-samples the circular-mean kernel evaluates
 };
 
-constexpr double kUnitOverhead = 24.0; // per-unit fixed cost, in angle iterations
+constexpr double kStageCost = 150.0;   // staging a tile, in angle iterations of each warp
+constexpr int kUnitsPerWarp = 1;       // units per warp from which on a plan uses more CTAs
+constexpr double kUnitOverhead = 6.0; // per-unit fixed cost, in angle iterations
 // Abel tiles of 64 from this many on (forward / adjoint time stage with tiles of
 // 32 and of 64: 10.8 / 10.9 and 12.7 / 11.8 us at 256^2, 128 detectors, 16
 // tiles of 64; 26.7 / 27.0 and 22 / 21 us at 512^2, 256 detectors, 64 tiles)
@@ -237,8 +239,6 @@ pat_status_t build_plan(Plan& P, const pat_geometry_t* geoms, int n_inst, const 
     P.geoms.assign(geoms, geoms + n_inst);
     P.opt = opt;
     const bool bf16 = opt.image_dtype == PAT_BF16;
-    const int ml = opt.m_lanes;
-    const int qpiece = opt.q_piece;
 
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return PAT_ERR_CUDA;
@@ -247,6 +247,22 @@ pat_status_t build_plan(Plan& P, const pat_geometry_t* geoms, int n_inst, const 
     if (cudaGetDeviceProperties(&prop, dev) != cudaSuccess) return PAT_ERR_CUDA;
     P.num_sms = prop.multiProcessorCount;
     P.max_smem_optin = (int)prop.sharedMemPerBlockOptin;
+    int ml = opt.m_lanes, qpiece = opt.q_piece;
+    {
+        // Radii per warp and angles per unit, where the options leave them open,
+        // by the warp steps (32 samples) per resident warp: a small plan needs
+        // many short units (whole forward with 32 radii and 128 angles / 8 and
+        // 64: 14.9 / 10.8 us at 64^2, 4 steps; 16 and 64: 16.8 / 14.7 us at
+        // 128^2, 15 steps), a large one few long ones (154 / 177 us at 512^2).
+        // About 41 % of a full circle's samples fall on the image.
+        double samples = 0.0;
+        for (int i = 0; i < n_inst; ++i)
+            samples += 0.41 * geoms[i].n_det * std::min(geoms[i].n_t + 2.0, 2.2 * geoms[i].n_t / geoms[i].t_max + 2.0) *
+                       geoms[i].n_angles;
+        const double steps = samples / (32.0 * P.num_sms * 2 * (kCircThreads / kWarp));
+        if (ml == 0) ml = steps < 8.0 ? 8 : steps < 50.0 ? 16 : 32;
+        if (qpiece == 0) qpiece = steps < 50.0 ? 64 : 128;
+    }
 
     // ---- offsets ----------------------------------------------------------
     P.f_offsets.assign(n_inst + 1, 0);
@@ -515,17 +531,29 @@ pat_status_t build_plan(Plan& P, const pat_geometry_t* geoms, int n_inst, const 
                 }
         for (int t = 0; t < ntiles; ++t) {
             auto& tile = T.tiles[t];
-            for (int j = 0; j < g.n_det; ++j) tile.units.insert(tile.units.end(), per[j][t].begin(), per[j][t].end());
+            // detectors in a scattered order (multiples of the golden section): a
+            // run of units then sees the tile from all sides.  Samples cost more or
+            // fewer bank conflicts by the direction of their rays, and a share of
+            // neighbouring detectors has only a few directions.
+            std::vector<std::pair<uint32_t, int>> jo;
+            for (int j = 0; j < g.n_det; ++j) jo.push_back({(uint32_t)j * 2654435769u, j});
+            std::sort(jo.begin(), jo.end());
+            for (const auto& x : jo) {
+                const auto& pu = per[x.second][t];
+                tile.units.insert(tile.units.end(), pu.begin(), pu.end());
+            }
             for (const Unit& u : tile.units) tile.cost += (double)(u.nq + QL - 1) / QL + kUnitOverhead;
         }
     }
 
     // ---- CTA schedule for the circular means ------------------------------
-    // Tile tasks: (instance, tile).  Each task gets CTAs ("parts") in
-    // proportion to its cost (at least one); parts are placed on CTAs by LPT.
-    // Within a task, the units are spread over the parts' warps by LPT on
-    // their cost (a sample costs the same everywhere), once per template tile
-    // and part count, so identical instances share the schedule.
+    // Tile tasks: (instance, tile).  The units of all tasks form one sequence
+    // that is cut into equal-cost shares, one per CTA; a CTA stages each tile
+    // that its share touches.  (Giving every tile a whole number of CTAs left
+    // them up to a quarter apart: at 512^2 the forward took 162 to 205 us,
+    // depending on the unit shape alone.)  A share's units of a tile are spread
+    // over its warps by LPT on their cost (a sample costs the same
+    // everywhere); whole tiles of identical instances share that list.
     const int64_t smem_bytes64 = tile_bytes + ray_bytes;
     if (smem_bytes64 > P.max_smem_optin) return PAT_ERR_UNSUPPORTED;
     const int smem_bytes = (int)smem_bytes64;
@@ -538,92 +566,100 @@ pat_status_t build_plan(Plan& P, const pat_geometry_t* geoms, int n_inst, const 
     double total_cost = 0.0;
     for (int i = 0; i < n_inst; ++i)
         for (const auto& tt : tmpls[inst_tmpl[i]].tiles) total_cost += tt.cost;
-    // parts per template tile
-    std::vector<std::vector<int>> tile_parts(tmpls.size());
-    for (size_t t = 0; t < tmpls.size(); ++t) {
-        tile_parts[t].resize(tmpls[t].tiles.size(), 0);
-        for (size_t k = 0; k < tmpls[t].tiles.size(); ++k) {
-            const TileTemplate& tt = tmpls[t].tiles[k];
-            if (tt.units.empty()) continue;
-            const double share = tt.cost / std::max(total_cost, 1.0) * n_ctas_target;
-            const int nunits = (int)tt.units.size();
-            tile_parts[t][k] = std::max(1, std::min((int)std::lround(share), std::max(1, nunits / (2 * kWarpsCta))));
-        }
-    }
-    // per (template tile): units grouped by (part, warp); offsets per warp
     std::vector<Unit> units;
-    std::vector<int32_t> warp_units;
-    std::vector<std::vector<int32_t>> tile_woff(tmpls.size());   // first warp_units index of (tile, part 0)
-    for (size_t t = 0; t < tmpls.size(); ++t) {
-        tile_woff[t].assign(tmpls[t].tiles.size(), -1);
-        for (size_t k = 0; k < tmpls[t].tiles.size(); ++k) {
-            const TileTemplate& tt = tmpls[t].tiles[k];
-            const int np = tile_parts[t][k];
-            if (np == 0) continue;
-            const int nw = np * kWarpsCta;
-            std::vector<std::vector<Unit>> lists(nw);
-            using E = std::pair<double, int>;
-            std::priority_queue<E, std::vector<E>, std::greater<E>> pq;
-            for (int w = 0; w < nw; ++w) pq.push({0.0, w});
-            for (const Unit& u : tt.units) {   // units are sorted largest first
-                E e = pq.top();
-                pq.pop();
-                lists[e.second].push_back(u);
-                pq.push({e.first + unit_cost(u), e.second});
-            }
-            tile_woff[t][k] = (int32_t)warp_units.size();
-            for (int w = 0; w < nw; ++w) {
-                warp_units.push_back((int32_t)units.size());
-                units.insert(units.end(), lists[w].begin(), lists[w].end());
-            }
-            warp_units.push_back((int32_t)units.size());   // end of the last warp (one slot per tile)
-        }
-    }
-    struct PartC {
-        Segment s;
-        double cost;
-    };
-    std::vector<PartC> parts;
-    for (int i = 0; i < n_inst; ++i) {
-        const int t = inst_tmpl[i];
-        const GeomTemplate& T = tmpls[t];
-        for (size_t k = 0; k < T.tiles.size(); ++k) {
-            const TileTemplate& tt = T.tiles[k];
-            const int np = tile_parts[t][k];
-            for (int p = 0; p < np; ++p) {
-                Segment s{};
-                s.inst = i;
-                s.x0 = tt.x0;
-                s.x1 = tt.x1;
-                s.y0 = tt.y0;
-                s.y1 = tt.y1;
-                s.pitch = cell_pitch(tt.x1 - tt.x0);
-                s.warp_off = tile_woff[t][k] + p * kWarpsCta;
-                parts.push_back({s, tt.cost / np});
-            }
-        }
-    }
-    std::stable_sort(parts.begin(), parts.end(), [](const PartC& a, const PartC& b) { return a.cost > b.cost; });
-    const int n_ctas = std::max(1, std::min(n_ctas_target, (int)parts.size()));
-    std::vector<std::vector<Segment>> cta_lists(n_ctas);
-    {
+    std::vector<int32_t> warp_units;   // per segment: the first unit of each warp, and the end
+    std::vector<std::pair<double, int>> order;
+    auto add_lists = [&](const TileTemplate& tt, size_t u0, size_t u1) {
+        order.clear();
+        for (size_t u = u0; u < u1; ++u) order.push_back({-unit_cost(tt.units[u]), (int)u});
+        std::sort(order.begin(), order.end());
+        std::vector<Unit> lists[kWarpsCta];
         using E = std::pair<double, int>;
         std::priority_queue<E, std::vector<E>, std::greater<E>> pq;
-        for (int c = 0; c < n_ctas; ++c) pq.push({0.0, c});
-        for (const PartC& p : parts) {
+        for (int w = 0; w < kWarpsCta; ++w) pq.push({0.0, w});
+        for (const auto& o : order) {   // largest first
             E e = pq.top();
             pq.pop();
-            cta_lists[e.second].push_back(p.s);
-            pq.push({e.first + p.cost + 8.0 * kUnitOverhead, e.second});
+            lists[e.second].push_back(tt.units[o.second]);
+            pq.push({e.first - o.first, e.second});
         }
-    }
+        const int32_t off = (int32_t)warp_units.size();
+        for (const auto& l : lists) {
+            warp_units.push_back((int32_t)units.size());
+            units.insert(units.end(), l.begin(), l.end());
+        }
+        warp_units.push_back((int32_t)units.size());
+        return off;
+    };
+    std::vector<std::vector<int32_t>> full_off(tmpls.size());   // warp_units index of a whole tile's lists
+    int64_t n_tasks = 0, n_units_all = 0;
+    for (size_t t = 0; t < tmpls.size(); ++t) full_off[t].assign(tmpls[t].tiles.size(), -1);
+    for (int i = 0; i < n_inst; ++i)
+        for (const auto& tt : tmpls[inst_tmpl[i]].tiles)
+            if (!tt.units.empty()) {
+                ++n_tasks;
+                n_units_all += (int64_t)tt.units.size();
+            }
+    const int n_ctas = (int)std::max<int64_t>(
+        1, std::min<int64_t>(n_ctas_target, n_units_all / (kWarpsCta * kUnitsPerWarp)));
     std::vector<Segment> segs;
     std::vector<int32_t> cta_seg(1, 0);
-    for (auto& l : cta_lists) {
-        segs.insert(segs.end(), l.begin(), l.end());
-        cta_seg.push_back((int32_t)segs.size());
+    {
+        const double stage = kStageCost * kWarpsCta;   // staging a tile, all warps
+        double left = total_cost + stage * (double)(n_tasks + n_ctas), load = 0.0;
+        int cta = 0;
+        double target = left / n_ctas;
+        auto next_cta = [&]() {
+            left -= load;
+            load = 0.0;
+            ++cta;
+            cta_seg.push_back((int32_t)segs.size());
+            target = left / (double)std::max(1, n_ctas - cta);
+        };
+        for (int i = 0; i < n_inst; ++i) {
+            const int t = inst_tmpl[i];
+            for (size_t k = 0; k < tmpls[t].tiles.size(); ++k) {
+                const TileTemplate& tt = tmpls[t].tiles[k];
+                size_t u0 = 0;
+                double rest = tt.cost;
+                while (u0 < tt.units.size()) {
+                    const bool last = cta == n_ctas - 1;
+                    double room = target - load - stage;
+                    if (!last && load > 0.0 && room < 0.05 * target) {
+                        next_cta();
+                        continue;
+                    }
+                    size_t u1 = tt.units.size();
+                    double c = rest;
+                    if (!last && rest > room + 0.03 * target) {
+                        room = std::max(room, 0.05 * target);
+                        c = 0.0;
+                        for (u1 = u0; u1 < tt.units.size() && (c < room || u1 == u0); ++u1) c += unit_cost(tt.units[u1]);
+                    }
+                    int32_t off;
+                    if (u0 == 0 && u1 == tt.units.size()) {
+                        if (full_off[t][k] < 0) full_off[t][k] = add_lists(tt, u0, u1);
+                        off = full_off[t][k];
+                    } else {
+                        off = add_lists(tt, u0, u1);
+                    }
+                    Segment s{};
+                    s.inst = i;
+                    s.x0 = tt.x0;
+                    s.x1 = tt.x1;
+                    s.y0 = tt.y0;
+                    s.y1 = tt.y1;
+                    s.pitch = cell_pitch(tt.x1 - tt.x0);
+                    s.warp_off = off;
+                    segs.push_back(s);
+                    load += stage + c;
+                    rest -= c;
+                    u0 = u1;
+                }
+            }
+        }
+        if ((int32_t)segs.size() > cta_seg.back()) cta_seg.push_back((int32_t)segs.size());
     }
-    if (parts.empty()) cta_seg.assign(1, 0);
     std::vector<int2> msum_rows;
     for (int i = 0; i < n_inst; ++i)
         for (int j = 0; j < geoms[i].n_det; ++j) msum_rows.push_back(make_int2(i, j));
