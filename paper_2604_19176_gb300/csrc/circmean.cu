@@ -137,8 +137,16 @@ __device__ __forceinline__ float sample(const unsigned char* __restrict__ smem, 
 #define PAT_DBG_ARG
 #endif
 
+// 64 registers: one CTA of 1024 threads per SM, or two of 512.  One large CTA
+// stages a tile of twice the area, so fewer samples are evaluated for two
+// tiles (1.22 instead of 1.32 per sample on the image at 512^2) and a ray table
+// serves twice the warps: forward 154 -> 140 us at 512^2, 403 -> 361 us at
+// 760^2, 1142 -> 1000 us at 1024^2.  Small plans keep two CTAs (64^2: 10.8
+// against 11.3 us).  Bound by the L1 data path (83 % of its peak at 760^2: a
+// sample's 16-byte cell takes a quarter warp per wavefront), with 68 % of the
+// issue slots used.
 template <int ML, typename T>
-__global__ void __launch_bounds__(kCircThreads, 2) k_circmean(DevPlan dp, const T* __restrict__ f)
+__global__ void __launch_bounds__(kCircThreads, 1) k_circmean(DevPlan dp, const T* __restrict__ f)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t bar[2];
@@ -302,7 +310,7 @@ cudaError_t launch_circmean(const DevPlan& dp, const void* f, cudaStream_t st, b
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(dp.n_fwd_ctas);
-    cfg.blockDim = dim3(kCircThreads);
+    cfg.blockDim = dim3(dp.circ_threads);
     cfg.dynamicSmemBytes = (size_t)dp.fwd_smem_bytes;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
@@ -319,7 +327,7 @@ cudaError_t launch_circmean(const DevPlan& dp, const void* f, cudaStream_t st, b
                       1, dp);
 }
 
-int circmean_blocks_per_sm(int m_lanes, bool bf16, int smem_bytes)
+int circmean_blocks_per_sm(int m_lanes, bool bf16, int threads, int smem_bytes)
 {
     const void* fn = circ_select(m_lanes, bf16);
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes) != cudaSuccess) {
@@ -327,7 +335,7 @@ int circmean_blocks_per_sm(int m_lanes, bool bf16, int smem_bytes)
         return 0;
     }
     int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, kCircThreads, smem_bytes) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, threads, smem_bytes) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }

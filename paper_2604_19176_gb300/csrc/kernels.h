@@ -8,7 +8,7 @@
 
 namespace patgpu {
 
-constexpr int kCircThreads = 512;   // threads per circular-mean CTA (16 warps)
+constexpr int kCircThreads = 1024;   // most threads of a circular-mean CTA (512 on small plans)
 
 // Launches fn<<<grid, block, smem, st>>>(args...) with programmatic stream
 // serialization (the kernel must call pdl_wait before it reads or writes
@@ -78,7 +78,7 @@ cudaError_t launch_count_samples(const DevPlan& dp, int inst_idx, int n_det, uns
 
 // Occupancy of the circular-mean kernel for the plan's tile shape, and of the
 // adjoint cell kernel (256-thread CTAs).
-int circmean_blocks_per_sm(int m_lanes, bool bf16, int smem_bytes);
+int circmean_blocks_per_sm(int m_lanes, bool bf16, int threads, int smem_bytes);
 int adj_cells_blocks_per_sm();
 // Resident CTAs per SM of the list gather: lm 0 = code lists, 1 = fraction
 // lists, 2 = run-pair code lists.

@@ -291,6 +291,7 @@ struct DevPlan {
                                    //   0 = compute mode
     int32_t adj_jblock;            // code lists: detectors per aligned block
     int32_t cell_blocks;           // CTAs of the adjoint cell kernel (8 warps each)
+    int32_t circ_threads;          // threads of a circular-mean CTA
     int32_t fwd_smem_bytes;        // dynamic shared memory of the circular-mean kernel
     int32_t fwd_rays_off;          // byte offset of the staged rays (after the largest tile)
     int32_t wait_probe;            // test hook: CTA 0 of the next circular-mean launch waits on a

@@ -247,7 +247,7 @@ pat_status_t build_plan(Plan& P, const pat_geometry_t* geoms, int n_inst, const 
     if (cudaGetDeviceProperties(&prop, dev) != cudaSuccess) return PAT_ERR_CUDA;
     P.num_sms = prop.multiProcessorCount;
     P.max_smem_optin = (int)prop.sharedMemPerBlockOptin;
-    int ml = opt.m_lanes, qpiece = opt.q_piece;
+    int ml = opt.m_lanes, qpiece = opt.q_piece, circ_threads = kCircThreads;
     {
         // Radii per warp and angles per unit, where the options leave them open,
         // by the warp steps (32 samples) per resident warp: a small plan needs
@@ -259,9 +259,14 @@ pat_status_t build_plan(Plan& P, const pat_geometry_t* geoms, int n_inst, const 
         for (int i = 0; i < n_inst; ++i)
             samples += 0.41 * geoms[i].n_det * std::min(geoms[i].n_t + 2.0, 2.2 * geoms[i].n_t / geoms[i].t_max + 2.0) *
                        geoms[i].n_angles;
-        const double steps = samples / (32.0 * P.num_sms * 2 * (kCircThreads / kWarp));
+        const double steps = samples / (32.0 * P.num_sms * (kCircThreads / kWarp));
         if (ml == 0) ml = steps < 8.0 ? 8 : steps < 50.0 ? 16 : 32;
         if (qpiece == 0) qpiece = steps < 50.0 ? 64 : 128;
+        // one large CTA per SM, or two (with half the shared memory each) on small plans
+        if (steps < 50.0) {
+            circ_threads = kCircThreads / 2;
+            P.band_budget_bytes = 110 * 1024;
+        }
     }
 
     // ---- offsets ----------------------------------------------------------
@@ -558,10 +563,10 @@ pat_status_t build_plan(Plan& P, const pat_geometry_t* geoms, int n_inst, const 
     if (smem_bytes64 > P.max_smem_optin) return PAT_ERR_UNSUPPORTED;
     const int smem_bytes = (int)smem_bytes64;
     P.fwd_smem = smem_bytes;
-    const int bps = circmean_blocks_per_sm(ml, bf16, smem_bytes);
+    const int bps = circmean_blocks_per_sm(ml, bf16, circ_threads, smem_bytes);
     if (bps < 1) return PAT_ERR_UNSUPPORTED;
     const int n_ctas_target = bps * P.num_sms;
-    constexpr int kWarpsCta = kCircThreads / kWarp;
+    const int warps_cta = circ_threads / kWarp;
     auto unit_cost = [&](const Unit& u) { return (double)((u.nq + QL - 1) / QL) + kUnitOverhead; };
     double total_cost = 0.0;
     for (int i = 0; i < n_inst; ++i)
@@ -573,10 +578,10 @@ pat_status_t build_plan(Plan& P, const pat_geometry_t* geoms, int n_inst, const 
         order.clear();
         for (size_t u = u0; u < u1; ++u) order.push_back({-unit_cost(tt.units[u]), (int)u});
         std::sort(order.begin(), order.end());
-        std::vector<Unit> lists[kWarpsCta];
+        std::vector<std::vector<Unit>> lists(warps_cta);
         using E = std::pair<double, int>;
         std::priority_queue<E, std::vector<E>, std::greater<E>> pq;
-        for (int w = 0; w < kWarpsCta; ++w) pq.push({0.0, w});
+        for (int w = 0; w < warps_cta; ++w) pq.push({0.0, w});
         for (const auto& o : order) {   // largest first
             E e = pq.top();
             pq.pop();
@@ -601,11 +606,11 @@ pat_status_t build_plan(Plan& P, const pat_geometry_t* geoms, int n_inst, const 
                 n_units_all += (int64_t)tt.units.size();
             }
     const int n_ctas = (int)std::max<int64_t>(
-        1, std::min<int64_t>(n_ctas_target, n_units_all / (kWarpsCta * kUnitsPerWarp)));
+        1, std::min<int64_t>(n_ctas_target, n_units_all / (warps_cta * kUnitsPerWarp)));
     std::vector<Segment> segs;
     std::vector<int32_t> cta_seg(1, 0);
     {
-        const double stage = kStageCost * kWarpsCta;   // staging a tile, all warps
+        const double stage = kStageCost * warps_cta;   // staging a tile, all warps
         double left = total_cost + stage * (double)(n_tasks + n_ctas), load = 0.0;
         int cta = 0;
         double target = left / n_ctas;
@@ -967,6 +972,7 @@ pat_status_t build_plan(Plan& P, const pat_geometry_t* geoms, int n_inst, const 
     dp.m_lanes = ml;
     dp.adj_groups = AG;
     dp.cell_blocks = cell_blocks;
+    dp.circ_threads = circ_threads;
     dp.fwd_smem_bytes = smem_bytes;
     dp.fwd_rays_off = (int32_t)tile_bytes;
     dp.abel_tile = abel_tile;
