@@ -363,12 +363,17 @@ __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory"); }
 } // namespace
 
-// DUAL = false: r = A f - g (y, if not null, receives r).
-// DUAL = true:  y <- (y + sigma (A f - g)) * inv1ps and r = the new y.
-template <bool DUAL>
+// kResidual: r = A f - g (y, if not null, receives r).
+// kDual:     y <- (y + sigma (A f - g)) * inv1ps and r = the new y.
+// kForward:  y <- A f, no adjoint (gdata unused): the time stage of pat_forward
+//            on the plans that the solver steps fuse, in one launch instead of
+//            the radius sums and k_abel.
+enum TimeMode { kResidual, kDual, kForward };
+template <TimeMode MODE>
 __global__ void __launch_bounds__(kTimeThreads, 2) k_time_pair(DevPlan dp, const float* __restrict__ gdata,
                                                               float* __restrict__ y, float sigma, float inv1ps)
 {
+    constexpr bool DUAL = MODE == kDual;
     extern __shared__ __align__(16) unsigned char tp_smem[];
     const int nch = dp.time_chunks;                                  // most chunks of a CTA in one phase
     float* Ms = reinterpret_cast<float*>(tp_smem);                   // [radius][detector]
@@ -460,7 +465,7 @@ __global__ void __launch_bounds__(kTimeThreads, 2) k_time_pair(DevPlan dp, const
     pdl_wait();   // the partial slots come from the circular-mean kernel; g and y from earlier work
 
     // the data (and y) of this CTA's time chunks, for the forward epilogue
-    for (int p = sub; time_chunk(p, rank) < n_tc; p += kTimeSub) {
+    for (int p = sub; MODE != kForward && time_chunk(p, rank) < n_tc; p += kTimeSub) {
         const int x = 32 * time_chunk(p, rank) + lane;
         const bool ok = jd < grp.jn && x < in.n_t;
         const size_t o = ok ? in.g_off + (size_t)(grp.j0 + jd) * in.n_t + x : 0;
@@ -517,6 +522,7 @@ __global__ void __launch_bounds__(kTimeThreads, 2) k_time_pair(DevPlan dp, const
         if (own != rank)
             reinterpret_cast<float4*>(Ms)[idx] = reinterpret_cast<const float4*>(cluster.map_shared_rank(Ms, own))[idx];
     }
+    if (MODE == kForward) cluster_arrive();   // this CTA has read the others' shared memory (waited for at exit)
     __syncthreads();
 
     // 2. forward blocks, then the CTA's time chunks: g = sum / K and the residual
@@ -536,7 +542,9 @@ __global__ void __launch_bounds__(kTimeThreads, 2) k_time_pair(DevPlan dp, const
             const float* d = gs + (size_t)(p * 2 * kTimeJ + jd) * kWarp + lane;
             const size_t o = in.g_off + (size_t)(grp.j0 + jd) * in.n_t + x;
             const float g = sum * in.inv_K;
-            if (DUAL) {
+            if (MODE == kForward) {
+                y[o] = g;
+            } else if (DUAL) {
                 r = fmaf(sigma, g - d[0], d[kTimeJ * kWarp]) * inv1ps;
                 y[o] = r;
             } else {
@@ -544,7 +552,11 @@ __global__ void __launch_bounds__(kTimeThreads, 2) k_time_pair(DevPlan dp, const
                 if (y) y[o] = r;
             }
         }
-        rs[x * kTimeJ + jd] = r;   // zero for absent detectors and padded times
+        if (MODE != kForward) rs[x * kTimeJ + jd] = r;   // zero for absent detectors and padded times
+    }
+    if (MODE == kForward) {
+        cluster_wait();   // no CTA leaves while another may still read its shared memory
+        return;
     }
 
     // 3. exchange of the residual chunks
@@ -575,14 +587,14 @@ __global__ void __launch_bounds__(kTimeThreads, 2) k_time_pair(DevPlan dp, const
 }
 
 namespace {
-template <bool DUAL>
+template <TimeMode MODE>
 cudaError_t launch_time_pair_t(const DevPlan& dp, const float* g, float* y, float sigma, float inv1ps,
                                cudaStream_t st)
 {
-    cudaError_t e = cudaFuncSetAttribute(k_time_pair<DUAL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(k_time_pair<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          dp.time_smem_bytes);
     if (e != cudaSuccess) return e;
-    return launch_pdl(k_time_pair<DUAL>, dim3((unsigned)(dp.n_time_groups * kTimeCS)), dim3(kTimeThreads),
+    return launch_pdl(k_time_pair<MODE>, dim3((unsigned)(dp.n_time_groups * kTimeCS)), dim3(kTimeThreads),
                       (size_t)dp.time_smem_bytes, st, kTimeCS, dp, g, y, sigma, inv1ps);
 }
 } // namespace
@@ -592,13 +604,20 @@ cudaError_t launch_time_pair(const DevPlan& dp, const float* g, float* y, bool d
 {
     if (dp.n_time_groups == 0) return cudaSuccess;
     if (dp.time_chunks <= 0) return cudaErrorInvalidValue;
-    return dual ? launch_time_pair_t<true>(dp, g, y, sigma, inv1ps, st)
-                : launch_time_pair_t<false>(dp, g, y, sigma, inv1ps, st);
+    return dual ? launch_time_pair_t<kDual>(dp, g, y, sigma, inv1ps, st)
+                : launch_time_pair_t<kResidual>(dp, g, y, sigma, inv1ps, st);
+}
+
+cudaError_t launch_time_fwd(const DevPlan& dp, float* g, cudaStream_t st)
+{
+    if (dp.n_time_groups == 0) return cudaSuccess;
+    if (dp.time_chunks <= 0) return cudaErrorInvalidValue;
+    return launch_time_pair_t<kForward>(dp, nullptr, g, 0.f, 1.f, st);
 }
 
 int time_pair_clusters(int smem_bytes)
 {
-    const void* fn = reinterpret_cast<const void*>(k_time_pair<false>);
+    const void* fn = reinterpret_cast<const void*>(k_time_pair<kResidual>);
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes) != cudaSuccess) {
         cudaGetLastError();
         return 0;

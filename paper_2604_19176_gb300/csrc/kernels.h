@@ -46,6 +46,8 @@ cudaError_t launch_abel_adj(const DevPlan& dp, const float* g, cudaStream_t st);
 // of the steps: Mbar from the circular-mean partial slots in one launch.
 cudaError_t launch_time_pair(const DevPlan& dp, const float* g, float* y, bool dual, float sigma, float inv1ps,
                              cudaStream_t st);
+// Its forward half alone (radius sums and forward): g = A f from the partial slots.
+cudaError_t launch_time_fwd(const DevPlan& dp, float* g, cudaStream_t st);
 // Clusters of the fused time stage that fit the GPU at once (0: cannot run).
 int time_pair_clusters(int smem_bytes);
 cudaError_t launch_adjoint_gather(const DevPlan& dp, void* f, cudaStream_t st);
