@@ -42,9 +42,17 @@ class Geometry:
                                 self.n_angles)
 
 
-def _stream_ptr(stream, device) -> ctypes.c_void_p:
-    s = stream if stream is not None else torch.cuda.current_stream(device)
-    return ctypes.c_void_p(s.cuda_stream)
+# A call of the smallest problem takes the host longer than the GPU, so a call
+# makes no object that the library does not need: pointers and the stream go to
+# the library as plain integers (the prototypes convert them), and the current
+# stream is asked for by its raw handle (0.1 instead of 2.2 us for a
+# torch.cuda.Stream object).
+def _stream_ptr(stream, device: torch.device) -> int:
+    return stream.cuda_stream if stream is not None else torch._C._cuda_getCurrentRawStream(device.index)
+
+
+def _ptr(t: torch.Tensor | None) -> int:
+    return 0 if t is None else t.data_ptr()
 
 
 class PatPlan:
@@ -94,6 +102,9 @@ class PatPlan:
         self.g_offsets = list(go)
         g0 = self.geoms[0]
         self.uniform = all(g == g0 for g in self.geoms)
+        batch = () if len(self.geoms) == 1 else (len(self.geoms),)
+        self._image_shape = (*batch, g0.n, g0.n) if self.uniform else (self.f_elems,)
+        self._data_shape = (*batch, g0.n_det, g0.n_t) if self.uniform else (self.g_elems,)
 
     # -- bookkeeping ---------------------------------------------------------
     def close(self) -> None:
@@ -134,18 +145,15 @@ class PatPlan:
         return self.g_offsets[-1]
 
     def image_shape(self) -> tuple[int, ...]:
-        g = self.geoms[0]
-        if not self.uniform:
-            return (self.f_elems,)
-        return (g.n, g.n) if len(self.geoms) == 1 else (len(self.geoms), g.n, g.n)
+        return self._image_shape
 
     def data_shape(self) -> tuple[int, ...]:
-        g = self.geoms[0]
-        if not self.uniform:
-            return (self.g_elems,)
-        return (g.n_det, g.n_t) if len(self.geoms) == 1 else (len(self.geoms), g.n_det, g.n_t)
+        return self._data_shape
 
     def _check(self, t: torch.Tensor, numel: int, dtype, name: str) -> None:
+        if (isinstance(t, torch.Tensor) and t.is_cuda and t.get_device() == self.device.index and t.dtype is dtype
+                and t.is_contiguous() and t.numel() == numel):
+            return
         if not isinstance(t, torch.Tensor) or t.device.type != "cuda":
             raise ValueError(f"{name} must be a CUDA tensor")
         if t.device.index != self.device.index:
@@ -160,10 +168,10 @@ class PatPlan:
         """g = A f (every instance)."""
         self._check(f, self.f_elems, self.image_dtype, "f")
         if out is None:
-            out = torch.empty(self.data_shape(), dtype=torch.float32, device=self.device)
-        self._check(out, self.g_elems, torch.float32, "out")
-        _lib.check("pat_forward", self._lib.pat_forward(self._h, ctypes.c_void_p(f.data_ptr()),
-                                                        ctypes.c_void_p(out.data_ptr()),
+            out = torch.empty(self._data_shape, dtype=torch.float32, device=self.device)
+        else:
+            self._check(out, self.g_elems, torch.float32, "out")
+        _lib.check("pat_forward", self._lib.pat_forward(self._h, f.data_ptr(), out.data_ptr(),
                                                         _stream_ptr(stream, self.device)))
         return out
 
@@ -171,10 +179,10 @@ class PatPlan:
         """f = A^T g (every instance)."""
         self._check(g, self.g_elems, torch.float32, "g")
         if out is None:
-            out = torch.empty(self.image_shape(), dtype=self.image_dtype, device=self.device)
-        self._check(out, self.f_elems, self.image_dtype, "out")
-        _lib.check("pat_adjoint", self._lib.pat_adjoint(self._h, ctypes.c_void_p(g.data_ptr()),
-                                                        ctypes.c_void_p(out.data_ptr()),
+            out = torch.empty(self._image_shape, dtype=self.image_dtype, device=self.device)
+        else:
+            self._check(out, self.f_elems, self.image_dtype, "out")
+        _lib.check("pat_adjoint", self._lib.pat_adjoint(self._h, g.data_ptr(), out.data_ptr(),
                                                         _stream_ptr(stream, self.device)))
         return out
 
@@ -184,19 +192,18 @@ class PatPlan:
         self._check(f, self.f_elems, torch.float32, "f")
         if grad is None:
             grad = torch.empty_like(f)
-        self._check(grad, self.f_elems, torch.float32, "grad")
+        else:
+            self._check(grad, self.f_elems, torch.float32, "grad")
         val = torch.empty(len(self.geoms), dtype=torch.float32, device=self.device) if want_value else None
         _lib.check("pat_tv_grad", self._lib.pat_tv_grad(
-            self._h, ctypes.c_void_p(f.data_ptr()), ctypes.c_float(eps), ctypes.c_void_p(grad.data_ptr()),
-            ctypes.c_void_p(val.data_ptr() if val is not None else 0), _stream_ptr(stream, self.device)))
+            self._h, f.data_ptr(), ctypes.c_float(eps), grad.data_ptr(), _ptr(val), _stream_ptr(stream, self.device)))
         return val, grad
 
     def tv_value(self, f: torch.Tensor, eps: float, stream=None) -> torch.Tensor:
         self._check(f, self.f_elems, torch.float32, "f")
         val = torch.empty(len(self.geoms), dtype=torch.float32, device=self.device)
         _lib.check("pat_tv_grad", self._lib.pat_tv_grad(
-            self._h, ctypes.c_void_p(f.data_ptr()), ctypes.c_float(eps), ctypes.c_void_p(0),
-            ctypes.c_void_p(val.data_ptr()), _stream_ptr(stream, self.device)))
+            self._h, f.data_ptr(), ctypes.c_float(eps), None, val.data_ptr(), _stream_ptr(stream, self.device)))
         return val
 
     def residual(self, Af: torch.Tensor, g: torch.Tensor, out: torch.Tensor | None = None, scale: float = 1.0,
@@ -206,10 +213,11 @@ class PatPlan:
         self._check(g, self.g_elems, torch.float32, "g")
         if out is None:
             out = torch.empty_like(Af)
-        self._check(out, self.g_elems, torch.float32, "out")
+        else:
+            self._check(out, self.g_elems, torch.float32, "out")
         _lib.check("pat_residual", self._lib.pat_residual(
-            self._h, ctypes.c_void_p(Af.data_ptr()), ctypes.c_void_p(g.data_ptr()), ctypes.c_void_p(out.data_ptr()),
-            ctypes.c_float(scale), _stream_ptr(stream, self.device)))
+            self._h, Af.data_ptr(), g.data_ptr(), out.data_ptr(), ctypes.c_float(scale),
+            _stream_ptr(stream, self.device)))
         return out
 
     def descent_step(self, f: torch.Tensor, adj: torch.Tensor, tvgrad: torch.Tensor | None, tau: float, lam: float,
@@ -222,10 +230,8 @@ class PatPlan:
         if delta is not None:
             self._check(delta, 2 * len(self.geoms), torch.float32, "delta")
         _lib.check("pat_descent_step", self._lib.pat_descent_step(
-            self._h, ctypes.c_void_p(f.data_ptr()), ctypes.c_void_p(adj.data_ptr()),
-            ctypes.c_void_p(tvgrad.data_ptr() if tvgrad is not None else 0), ctypes.c_float(tau),
-            ctypes.c_float(lam), 1 if nonneg else 0, ctypes.c_void_p(delta.data_ptr() if delta is not None else 0),
-            _stream_ptr(stream, self.device)))
+            self._h, f.data_ptr(), adj.data_ptr(), _ptr(tvgrad), ctypes.c_float(tau), ctypes.c_float(lam),
+            1 if nonneg else 0, _ptr(delta), _stream_ptr(stream, self.device)))
 
     def tv_step(self, f_in: torch.Tensor, f_out: torch.Tensor, g: torch.Tensor, tau: float, lam: float, eps: float,
                 nonneg: bool = True, delta: torch.Tensor | None = None, stream=None) -> None:
@@ -236,10 +242,8 @@ class PatPlan:
         if delta is not None:
             self._check(delta, 2 * len(self.geoms), torch.float32, "delta")
         _lib.check("pat_tv_step", self._lib.pat_tv_step(
-            self._h, ctypes.c_void_p(f_in.data_ptr()), ctypes.c_void_p(f_out.data_ptr()),
-            ctypes.c_void_p(g.data_ptr()), ctypes.c_float(tau), ctypes.c_float(lam), ctypes.c_float(eps),
-            1 if nonneg else 0, ctypes.c_void_p(delta.data_ptr() if delta is not None else 0),
-            _stream_ptr(stream, self.device)))
+            self._h, f_in.data_ptr(), f_out.data_ptr(), g.data_ptr(), ctypes.c_float(tau), ctypes.c_float(lam),
+            ctypes.c_float(eps), 1 if nonneg else 0, _ptr(delta), _stream_ptr(stream, self.device)))
 
     def pdhg_step(self, f: torch.Tensor, fbar: torch.Tensor, y: torch.Tensor, px: torch.Tensor, py: torch.Tensor,
                   g: torch.Tensor, sigma: float, tau: float, alpha: float, nonneg: bool = True,
@@ -256,11 +260,10 @@ class PatPlan:
             self._check(delta, 2 * len(self.geoms), torch.float32, "delta")
         if fmean is not None:
             self._check(fmean, len(self.geoms), torch.float32, "fmean")
-        ptr = lambda t: ctypes.c_void_p(t.data_ptr() if t is not None else 0)  # noqa: E731
         _lib.check("pat_pdhg_step", self._lib.pat_pdhg_step(
-            self._h, ptr(f), ptr(fbar), ptr(y), ptr(px), ptr(py), ptr(g), ctypes.c_float(sigma), ctypes.c_float(tau),
-            ctypes.c_float(alpha), 1 if nonneg else 0, ctypes.c_float(beta), ctypes.c_float(mean_target), ptr(fmean),
-            ptr(delta), _stream_ptr(stream, self.device)))
+            self._h, f.data_ptr(), fbar.data_ptr(), y.data_ptr(), px.data_ptr(), py.data_ptr(), g.data_ptr(),
+            ctypes.c_float(sigma), ctypes.c_float(tau), ctypes.c_float(alpha), 1 if nonneg else 0, ctypes.c_float(beta),
+            ctypes.c_float(mean_target), _ptr(fmean), _ptr(delta), _stream_ptr(stream, self.device)))
 
     def set_timing(self, enable: bool) -> None:
         """Bracket every kernel launch of this plan with CUDA events."""
