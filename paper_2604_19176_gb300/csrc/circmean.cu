@@ -86,17 +86,35 @@ struct UnitFrame {
     uint32_t lim;   // debug builds: largest valid byte offset of a staged cell
 };
 
-__device__ __forceinline__ UnitFrame unit_frame(const Segment& sg, const InstDev& in, float4 d)
+__device__ __forceinline__ UnitFrame unit_frame(const Segment& sg, const InstDev& in, const Unit& un)
 {
     UnitFrame u;
-    const int Ui = __float2int_rz(d.x), Vi = __float2int_rz(d.y);
     // staged column index = floor + Ui + c0 - (x0 - 2); bits = kMagicBits + floor
-    u.ulo = kMagicBits + (uint32_t)(sg.x0 - 2 - Ui - in.c0);
-    u.vlo = kMagicBits + (uint32_t)(sg.y0 - 2 - Vi - in.c0);
+    u.ulo = kMagicBits + (uint32_t)(sg.x0 - 2 - un.ui - in.c0);
+    u.vlo = kMagicBits + (uint32_t)(sg.y0 - 2 - un.vi - in.c0);
     u.uhi = u.ulo + (uint32_t)(sg.x1 - sg.x0 + 2);
     u.vhi = u.vlo + (uint32_t)(sg.y1 - sg.y0 + 2);
     u.row_bytes = (uint32_t)sg.pitch * 16u;
     u.koff = 0u - (u.vlo * u.row_bytes + u.ulo * 16u);   // modulo 2^32
+    return u;
+}
+
+// A unit's record from its eight words, held by lanes 0 to 7 (so a record in
+// flight takes one register of a warp that has none to spare).
+__device__ __forceinline__ Unit unit_of(int32_t word)
+{
+    auto w = [&](int i) { return __shfl_sync(0xffffffffu, word, i); };
+    Unit u;
+    u.j = w(0);
+    u.m0 = w(1);
+    u.q0 = w(2);
+    u.nq = w(3);
+    u.slot = w(4);
+    const int32_t uv = w(5);
+    u.ui = (int16_t)(uv & 0xffff);
+    u.vi = (int16_t)(uv >> 16);
+    u.uf = __int_as_float(w(6));
+    u.vf = __int_as_float(w(7));
     return u;
 }
 
@@ -142,9 +160,9 @@ __device__ __forceinline__ float sample(const unsigned char* __restrict__ smem, 
 // tiles (1.22 instead of 1.32 per sample on the image at 512^2) and a ray table
 // serves twice the warps: forward 154 -> 140 us at 512^2, 403 -> 361 us at
 // 760^2, 1142 -> 1000 us at 1024^2.  Small plans keep two CTAs (64^2: 10.8
-// against 11.3 us).  Bound by the L1 data path (83 % of its peak at 760^2: a
-// sample's 16-byte cell takes a quarter warp per wavefront), with 68 % of the
-// issue slots used.
+// against 11.3 us).  Bound by the L1 data path (93 % of its peak at 760^2: a
+// sample's 16-byte cell takes a quarter warp per wavefront), with 70 % of the
+// issue slots used; the SMs end within 3 % of each other.
 template <int ML, typename T>
 __global__ void __launch_bounds__(kCircThreads, 1) k_circmean(DevPlan dp, const T* __restrict__ f)
 {
@@ -183,6 +201,9 @@ __global__ void __launch_bounds__(kCircThreads, 1) k_circmean(DevPlan dp, const 
             mbar_arrive_expect_tx(&bar[0], ray_bytes);
             bulk_g2s(rays_s, dp.rays + in.ray_off, ray_bytes, &bar[0]);
         }
+        const int ub = dp.warp_units[sg.warp_off + warp], ue = dp.warp_units[sg.warp_off + warp + 1];
+        const int32_t* rec = reinterpret_cast<const int32_t*>(dp.units) + (lane & 7);
+        int32_t word = ub < ue ? rec[(size_t)ub * 8] : 0;
         if (tidx == task_begin) pdl_wait();   // f belongs to earlier work in the stream
         stage_cells(cells, f + in.f_off, in.n, sg);
         __syncthreads();
@@ -197,28 +218,21 @@ __global__ void __launch_bounds__(kCircThreads, 1) k_circmean(DevPlan dp, const 
         }
 
         // ---- this warp's units (static schedule) ------------------------------
-        const float4* det = dp.det + in.det_off;
         const size_t plane = (size_t)in.n_det * in.n_r;
         float* mpart = dp.mpart + in.mpart_off;
-        const int ub = dp.warp_units[sg.warp_off + warp], ue = dp.warp_units[sg.warp_off + warp + 1];
-        Unit un{};
-        if (ub < ue) un = dp.units[ub];
         for (int ui = ub; ui < ue; ++ui) {
-            Unit un2{};
-            if (ui + 1 < ue) un2 = dp.units[ui + 1];   // the next unit's record, in flight meanwhile
+            const Unit un = unit_of(word);
+            if (ui + 1 < ue) word = rec[(size_t)(ui + 1) * 8];   // the next unit's record, in flight meanwhile
             if (!dbg_ok(dp, un.j >= 0 && un.j < in.n_det && un.q0 >= 0 && un.nq >= 0 && un.q0 + un.nq <= in.K &&
                                 un.slot >= 0 && un.slot < in.n_slots && un.m0 >= 0,
-                        kSiteCircUnit)) {
-                un = un2;
+                        kSiteCircUnit))
                 continue;
-            }
             const int m = un.m0 + ml;
             const float mf = (float)m;
-            const float4 d = __ldg(det + un.j);
-            UnitFrame fr = unit_frame(sg, in, d);
+            UnitFrame fr = unit_frame(sg, in, un);
             fr.lim = (uint32_t)((sg.y1 - sg.y0 + 3) * sg.pitch - 1) * 16u;
             const float4* tq = rays_s + un.q0 + ql;   // units never wrap past K
-            const unsigned long long m2 = f2_pack(mf, mf), f0 = f2_pack(d.z, d.w);
+            const unsigned long long m2 = f2_pack(mf, mf), f0 = f2_pack(un.uf, un.vf);
             float acc0 = 0.f, acc1 = 0.f, acc2 = 0.f, acc3 = 0.f;
             int i = ql;
             for (; i + 3 * QL < un.nq; i += 4 * QL, tq += 4 * QL) {
@@ -233,7 +247,6 @@ __global__ void __launch_bounds__(kCircThreads, 1) k_circmean(DevPlan dp, const 
 #pragma unroll
             for (int o = ML; o < kWarp; o <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
             if (ql == 0 && m < in.n_r) mpart[(size_t)un.slot * plane + (size_t)un.j * in.n_r + m] = acc;
-            un = un2;
         }
     }
 }

@@ -78,9 +78,13 @@ struct InstDev {
 // Circular-mean work unit: radii [m0, m0 + m_lanes) of detector j, angles
 // q0 .. q0 + nq - 1 (never past K), restricted to one tile; its partial sums
 // go to forward slot `slot` (the slots of a (detector, radius block) are
-// added in slot order by k_msum).  32 bytes.
+// added in slot order by k_msum), and the detector's position in the split
+// form (integer and fractional parts), which the kernel would else wait for
+// once the record is there.  32 bytes.
 struct Unit {
-    int32_t j, m0, q0, nq, slot, pad[3];
+    int32_t j, m0, q0, nq, slot;
+    int16_t ui, vi;
+    float uf, vf;
 };
 
 // Tile task of the circular means: the pixels [x0, x1) x [y0, y1) of one

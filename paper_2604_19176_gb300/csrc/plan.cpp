@@ -158,9 +158,9 @@ struct GeomTemplate {
     int64_t slot_samples = 0;        // lane-samples the circular-mean kernel evaluates
 };
 
-constexpr double kStageCost = 150.0;   // staging a tile, in angle iterations of each warp
+constexpr double kStageCost = 60.0;    // staging a tile, in angle iterations of each warp (30 to 150: within 1 %)
 constexpr int kUnitsPerWarp = 1;       // units per warp from which on a plan uses more CTAs
-constexpr double kUnitOverhead = 6.0; // per-unit fixed cost, in angle iterations
+constexpr double kUnitOverhead = 3.0;  // per-unit fixed cost, in angle iterations (at 10: 3 % slower at 1024^2)
 // Abel tiles of 64 from this many on (forward / adjoint time stage with tiles of
 // 32 and of 64: 10.8 / 10.9 and 12.7 / 11.8 us at 256^2, 128 detectors, 16
 // tiles of 64; 26.7 / 27.0 and 22 / 21 us at 512^2, 256 detectors, 64 tiles)
@@ -473,6 +473,7 @@ pat_status_t build_plan(Plan& P, const pat_geometry_t* geoms, int n_inst, const 
         parallel_for(g.n_det, [&](int j) {
             std::vector<int> last(ntiles), start(ntiles);
             std::vector<std::vector<std::pair<int, int>>> runs(ntiles);   // [q_begin, q_end)
+            const float4 dj = det4[d.det_off + j];
             for (int mb = 0; mb < d.nmb; ++mb) {
                 const int m0 = mb * ml, m1 = std::min(m0 + ml, d.n_r) - 1;
                 const double r0 = m0 * delta, r1 = m1 * delta;
@@ -516,6 +517,10 @@ pat_status_t build_plan(Plan& P, const pat_geometry_t* geoms, int n_inst, const 
                             u.m0 = m0;
                             u.q0 = qs;
                             u.nq = piece;
+                            u.ui = (int16_t)dj.x;
+                            u.vi = (int16_t)dj.y;
+                            u.uf = dj.z;
+                            u.vf = dj.w;
                             per[j][t].push_back(u);
                             q0 += piece;
                             len -= piece;
@@ -556,7 +561,11 @@ pat_status_t build_plan(Plan& P, const pat_geometry_t* geoms, int n_inst, const 
     // that is cut into equal-cost shares, one per CTA; a CTA stages each tile
     // that its share touches.  (Giving every tile a whole number of CTAs left
     // them up to a quarter apart: at 512^2 the forward took 162 to 205 us,
-    // depending on the unit shape alone.)  A share's units of a tile are spread
+    // depending on the unit shape alone.  Cutting by the mean of what was left,
+    // with every boundary counted as one more staging, left the last of the CTAs
+    // without work: 145 of 152 had some at 256^2; the smallest share size that
+    // the CTAs suffice for took the forward from 27.2 to 25.5 us there, 361 to
+    // 334 us at 760^2, 996 to 957 us at 1024^2.)  A share's units of a tile are spread
     // over its warps by LPT on their cost (a sample costs the same
     // everywhere); whole tiles of identical instances share that list.
     const int64_t smem_bytes64 = tile_bytes + ray_bytes;
@@ -607,64 +616,75 @@ pat_status_t build_plan(Plan& P, const pat_geometry_t* geoms, int n_inst, const 
             }
     const int n_ctas = (int)std::max<int64_t>(
         1, std::min<int64_t>(n_ctas_target, n_units_all / (warps_cta * kUnitsPerWarp)));
-    std::vector<Segment> segs;
-    std::vector<int32_t> cta_seg(1, 0);
-    {
-        const double stage = kStageCost * warps_cta;   // staging a tile, all warps
-        double left = total_cost + stage * (double)(n_tasks + n_ctas), load = 0.0;
+    // cut(T, emit): the shares of at most T, in order; returns their number.  A
+    // tile's last units join a share that they exceed by less than 0.03 T, and
+    // no share takes less than 0.05 T of a tile.
+    const double stage = kStageCost * warps_cta;   // staging a tile, all warps
+    std::vector<std::vector<std::vector<double>>> before(tmpls.size());   // cost of a tile's units before each
+    for (size_t t = 0; t < tmpls.size(); ++t)
+        for (const auto& tt : tmpls[t].tiles) {
+            std::vector<double> b(1, 0.0);
+            for (const Unit& u : tt.units) b.push_back(b.back() + unit_cost(u));
+            before[t].push_back(std::move(b));
+        }
+    auto cut = [&](double target, auto&& emit) {
         int cta = 0;
-        double target = left / n_ctas;
-        auto next_cta = [&]() {
-            left -= load;
-            load = 0.0;
-            ++cta;
-            cta_seg.push_back((int32_t)segs.size());
-            target = left / (double)std::max(1, n_ctas - cta);
-        };
+        double load = 0.0;
         for (int i = 0; i < n_inst; ++i) {
             const int t = inst_tmpl[i];
             for (size_t k = 0; k < tmpls[t].tiles.size(); ++k) {
-                const TileTemplate& tt = tmpls[t].tiles[k];
-                size_t u0 = 0;
-                double rest = tt.cost;
-                while (u0 < tt.units.size()) {
-                    const bool last = cta == n_ctas - 1;
+                const std::vector<double>& b = before[t][k];
+                const size_t end = b.size() - 1;
+                for (size_t u0 = 0; u0 < end;) {
                     double room = target - load - stage;
-                    if (!last && load > 0.0 && room < 0.05 * target) {
-                        next_cta();
+                    if (load > 0.0 && room < 0.05 * target) {
+                        ++cta;
+                        load = 0.0;
                         continue;
                     }
-                    size_t u1 = tt.units.size();
-                    double c = rest;
-                    if (!last && rest > room + 0.03 * target) {
+                    size_t u1 = end;
+                    if (b[end] - b[u0] > room + 0.03 * target) {
                         room = std::max(room, 0.05 * target);
-                        c = 0.0;
-                        for (u1 = u0; u1 < tt.units.size() && (c < room || u1 == u0); ++u1) c += unit_cost(tt.units[u1]);
+                        u1 = std::lower_bound(b.begin() + u0 + 1, b.begin() + end, b[u0] + room) - b.begin();
                     }
-                    int32_t off;
-                    if (u0 == 0 && u1 == tt.units.size()) {
-                        if (full_off[t][k] < 0) full_off[t][k] = add_lists(tt, u0, u1);
-                        off = full_off[t][k];
-                    } else {
-                        off = add_lists(tt, u0, u1);
-                    }
-                    Segment s{};
-                    s.inst = i;
-                    s.x0 = tt.x0;
-                    s.x1 = tt.x1;
-                    s.y0 = tt.y0;
-                    s.y1 = tt.y1;
-                    s.pitch = cell_pitch(tt.x1 - tt.x0);
-                    s.warp_off = off;
-                    segs.push_back(s);
-                    load += stage + c;
-                    rest -= c;
+                    emit(cta, i, t, k, u0, u1);
+                    load += stage + b[u1] - b[u0];
                     u0 = u1;
                 }
             }
         }
-        if ((int32_t)segs.size() > cta_seg.back()) cta_seg.push_back((int32_t)segs.size());
+        return cta + 1;
+    };
+    // the smallest target that n_ctas shares are enough for
+    double lo = total_cost / n_ctas, hi = (total_cost + stage * (double)n_tasks) / 0.95;
+    for (int it = 0; it < 40 && hi - lo > 1e-4 * hi; ++it) {
+        const double mid = 0.5 * (lo + hi);
+        if (cut(mid, [](int, int, int, size_t, size_t, size_t) {}) <= n_ctas) hi = mid;
+        else lo = mid;
     }
+    std::vector<Segment> segs;
+    std::vector<int32_t> cta_seg(1, 0);
+    cut(hi, [&](int cta, int i, int t, size_t k, size_t u0, size_t u1) {
+        const TileTemplate& tt = tmpls[t].tiles[k];
+        while ((int)cta_seg.size() <= cta) cta_seg.push_back((int32_t)segs.size());
+        int32_t off;
+        if (u0 == 0 && u1 == tt.units.size()) {
+            if (full_off[t][k] < 0) full_off[t][k] = add_lists(tt, u0, u1);
+            off = full_off[t][k];
+        } else {
+            off = add_lists(tt, u0, u1);
+        }
+        Segment s{};
+        s.inst = i;
+        s.x0 = tt.x0;
+        s.x1 = tt.x1;
+        s.y0 = tt.y0;
+        s.y1 = tt.y1;
+        s.pitch = cell_pitch(tt.x1 - tt.x0);
+        s.warp_off = off;
+        segs.push_back(s);
+    });
+    if (!segs.empty()) cta_seg.push_back((int32_t)segs.size());
     std::vector<int2> msum_rows;
     for (int i = 0; i < n_inst; ++i)
         for (int j = 0; j < geoms[i].n_det; ++j) msum_rows.push_back(make_int2(i, j));
