@@ -304,7 +304,8 @@ struct DevPlan {
                                    //   out-of-range detector index for its bounds check to report
     int64_t n_code_vecs;           // adjoint lists: 16-byte vectors in the codes buffer
     int64_t n_win_vecs;            // windowed lists: code vectors (256 bytes each); 0 = not in use
-    int32_t win_n_warps[3];        //   warps of the launches for groups of four, two and one
+    int32_t win_n_warps[3];        //   warps (a share each) of the launches for groups of four, two and one
+    int32_t win_n_tail[3];         //   and the shares after those, which the warps take from a queue
     int32_t list_tail0;            // adjoint lists: list_items[list_tail0 ..] is the shared tail queue
     int32_t n_tail_items;          //   of small items (largest first), after the per-warp items
     int32_t abel_tile;             // side of the Abel tiles, 64 or 32

@@ -163,8 +163,9 @@ __device__ __forceinline__ float lds32(uint32_t addr)
 
 // 20 warps per SM (96 registers; 16 for four images): 24 warps at 80 registers
 // took 150 instead of 144 us at 512^2, and left L1 too little room.
-template <int NB>
-__global__ void __launch_bounds__(kWinThreads, NB == 4 ? 4 : 5) k_adj_win(DevPlan dp, int warp0, int n_warps)
+template <int NB, bool TAIL>
+__global__ void __launch_bounds__(kWinThreads, NB == 4 ? 4 : 5)
+    k_adj_win(DevPlan dp, int share0, int n_warps, int n_tail)
 {
     extern __shared__ __align__(16) unsigned char win_smem[];
     const int lane = threadIdx.x & 31;
@@ -180,7 +181,7 @@ __global__ void __launch_bounds__(kWinThreads, NB == 4 ? 4 : 5) k_adj_win(DevPla
         pdl_wait();
         return;
     }
-    const WinShare sh = dp.win_shares[warp0 + wid];
+    WinShare sh = dp.win_shares[share0 + wid];
     int gi = sh.group, bi = sh.block, part = sh.part;
     for (int i = lane; i < 8 * NB; i += kWarp) s_m[(i >> 3) * win_slots(NB) + (i & 7)] = 0.f;
 
@@ -213,6 +214,7 @@ __global__ void __launch_bounds__(kWinThreads, NB == 4 ? 4 : 5) k_adj_win(DevPla
         cp += 64;
     };
     start(bi, sh.ray_rec, sh.slot_rec, sh.code);
+    int32_t* const queue = dp.work_counters + kQueueStride;
     float4 tot[2][NB];   // moments of the two halves' cells over the blocks
     auto clear_totals = [&]() {
 #pragma unroll
@@ -220,8 +222,9 @@ __global__ void __launch_bounds__(kWinThreads, NB == 4 ? 4 : 5) k_adj_win(DevPla
     };
     clear_totals();
 #ifdef PAT_DEBUG
-    bool plant = dp.bounds_probe != 0 && blockIdx.x == 0 && warp0 == 0 && threadIdx.x == 0;
+    bool plant = dp.bounds_probe != 0 && blockIdx.x == 0 && share0 == 0 && threadIdx.x == 0;
 #endif
+    int ticket = wid;
     for (int k = 0; k < sh.count; ++k) {
         const WinGroup* G = dp.win_groups + gi;
         const int patch = (int)head.x;
@@ -266,8 +269,9 @@ __global__ void __launch_bounds__(kWinThreads, NB == 4 ? 4 : 5) k_adj_win(DevPla
             }
         }
         if (k == 0) {   // Mbar comes from the previous kernel, the rays from plan tables
-            pdl_wait();
+            if (!TAIL || ticket == wid) pdl_wait();
             stage_weights();
+            if (TAIL && lane == 0) ticket = n_warps + atomicAdd(queue, 1);
         }
         // ---- the next block's head and records, in flight while this one is processed
         const bool more = k + 1 < sh.count;
@@ -451,7 +455,20 @@ __global__ void __launch_bounds__(kWinThreads, NB == 4 ? 4 : 5) k_adj_win(DevPla
             const WinGroup* N = dp.win_groups + ++gi;
             start(0, N->ray_rec0, N->slot_rec0, N->code0);
         }
+        if constexpr (TAIL) {   // the next share from the queue
+            if (k + 1 < sh.count) continue;
+            ticket = __shfl_sync(0xffffffffu, ticket, 0);
+            if (ticket >= n_warps + n_tail) break;
+            sh = dp.win_shares[share0 + ticket];
+            gi = sh.group;
+            bi = sh.block;
+            part = sh.part;
+            start(bi, sh.ray_rec, sh.slot_rec, sh.code);
+            k = -1;
+        }
     }
+    // the last warp to run out of shares re-arms the queue for the next launch
+    if (TAIL && lane == 0 && atomicAdd(queue + 1, 1) == n_warps - 1) queue[0] = queue[1] = 0;
 }
 
 // ---------------------------------------------------------------------------
@@ -785,9 +802,9 @@ __global__ void __launch_bounds__(64) k_win_lists(DevPlan dp, int inst_idx, WinB
 namespace {
 const void* win_fn(int nb)
 {
-    return nb == 4   ? reinterpret_cast<const void*>(k_adj_win<4>)
-           : nb == 2 ? reinterpret_cast<const void*>(k_adj_win<2>)
-                     : reinterpret_cast<const void*>(k_adj_win<1>);
+    return nb == 4   ? reinterpret_cast<const void*>(k_adj_win<4, false>)
+           : nb == 2 ? reinterpret_cast<const void*>(k_adj_win<2, false>)
+                     : reinterpret_cast<const void*>(k_adj_win<1, false>);
 }
 int win_smem_bytes(int nb) { return (kWinThreads / kWarp) * win_warp_bytes(nb) + (int)kWinAlign - 16; }
 } // namespace
@@ -810,18 +827,21 @@ int adj_win_blocks_per_sm(int nb)
 
 cudaError_t launch_adj_win(const DevPlan& dp, cudaStream_t st)
 {
-    int warp0 = 0;
-    for (int c = 0; c < 3; ++c) {   // groups of 4, 2 and 1 instances
-        const int n = dp.win_n_warps[c], nb = c == 0 ? 4 : c == 1 ? 2 : 1;
+    int share0 = 0;
+    for (int c = 0; c < 3; ++c) {   // groups of 4, 2 and 1 images
+        const int n = dp.win_n_warps[c], tail = dp.win_n_tail[c], nb = c == 0 ? 4 : c == 1 ? 2 : 1;
         if (n == 0) continue;
         const int warps = kWinThreads / kWarp;
         const size_t smem = (size_t)win_smem_bytes(nb);
-        auto* fn = c == 0 ? k_adj_win<4> : c == 1 ? k_adj_win<2> : k_adj_win<1>;
+        auto* fn = c == 0   ? (tail ? k_adj_win<4, true> : k_adj_win<4, false>)
+                   : c == 1 ? (tail ? k_adj_win<2, true> : k_adj_win<2, false>)
+                            : (tail ? k_adj_win<1, true> : k_adj_win<1, false>);
         cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e == cudaSuccess)
-            e = launch_pdl(fn, dim3((n + warps - 1) / warps), dim3(kWinThreads), smem, st, 1, dp, warp0, n);
+            e = launch_pdl(fn, dim3((n + warps - 1) / warps), dim3(kWinThreads), smem, st, 1, dp, share0, n,
+                           tail);
         if (e != cudaSuccess) return e;
-        warp0 += n;
+        share0 += n + tail;
     }
     return cudaSuccess;
 }

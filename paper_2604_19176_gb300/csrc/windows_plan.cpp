@@ -48,6 +48,16 @@ double block_cost(const WinBlock& b, int nb)
     for (const uint2& h : b.half) c += 2.0 * (pair * (double)(h.y & 0xffffu) + one * (double)(h.y >> 16)) + 20.0;
     return c;
 }
+// Warps differ in what an instruction costs them (bank conflicts go by the
+// directions of their rays), so on plans with this many instructions per warp
+// the last quarter of the work is cut into small shares that the warps take
+// from a queue as they run out.  Gather without and with it: 5343 and 4775 us
+// for 8 x 1024^2, 1983 and 1761 us for 64 uneven instances, 1437 and 1379 us
+// for one 1024^2 image with single-image lists.  Below, a share that takes
+// some 8000 cycles to begin and to end is no longer small: 139 and 165 us at
+// 512^2, 341 and 356 us at 760^2.  Shares of 0.15 of a warp's mean instead of
+// 0.05: 4918 us for 8 x 1024^2; a tail of 0.15 or 0.4 of the work: 5044, 4810.
+constexpr double kTailFrom = 1e5, kTailPart = 0.25, kTailShare = 0.05;
 constexpr double kFlushCost = 100.0;   // end of a patch, per instance
 
 constexpr double kPatchRays = 11.0;   // rays of a detector that an 8 x 8 patch sees, about
@@ -312,7 +322,7 @@ pat_status_t build_windows(Plan& P, std::vector<InstDev>& inst, const std::vecto
         }
         const int g1 = (int)groups.size();
         if (n_tiles > INT32_MAX) return PAT_ERR_UNSUPPORTED;
-        dp.win_n_warps[cls] = 0;
+        dp.win_n_warps[cls] = dp.win_n_tail[cls] = 0;
         if (g0 == g1) continue;
         const int bps = adj_win_blocks_per_sm(nb);
         if (bps < 1) return PAT_ERR_UNSUPPORTED;
@@ -326,7 +336,11 @@ pat_status_t build_windows(Plan& P, std::vector<InstDev>& inst, const std::vecto
         for (int g = g0; g < g1; ++g)
             for (int b = 0; b < groups[g].n_blocks; ++b, ++seq) total += cost_of(groups[g], b);
         const int64_t n = std::min<int64_t>((int64_t)bps * P.num_sms * (kWinThreads / kWarp), seq);
-        const double share = total / (double)n;
+        const double tail_part = total / (double)n >= kTailFrom ? kTailPart : 0.0;
+        const double share = (1.0 - tail_part) * total / (double)n, tail_share = kTailShare * total / (double)n;
+        auto begin_at = [&](int64_t k) {   // cost before share k
+            return k <= n ? share * (double)k : share * (double)n + tail_share * (double)(k - n);
+        };
         double done = 0.0;
         int64_t k = 0;   // shares begun
         int last_patch = -1, last_group = -1;
@@ -334,7 +348,7 @@ pat_status_t build_windows(Plan& P, std::vector<InstDev>& inst, const std::vecto
             for (int b = 0; b < groups[g].n_blocks; ++b) {
                 const double c = cost_of(groups[g], b);
                 // a block belongs to the share that its middle falls into
-                const bool begin = k == 0 || (k < n && done + 0.5 * c >= share * (double)k);
+                const bool begin = k == 0 || ((k < n || tail_part > 0.0) && done + 0.5 * c >= begin_at(k));
                 const int patch = blocks[groups[g].block0 + b].patch;
                 int2& z = zinfo[groups[g].zinfo_off + patch];
                 const bool fresh = g != last_group || patch != last_patch;
@@ -349,8 +363,8 @@ pat_status_t build_windows(Plan& P, std::vector<InstDev>& inst, const std::vecto
                     *parts_max = std::max(*parts_max, z.y);
                 }
                 if (begin) {
+                    ++(k < n ? dp.win_n_warps : dp.win_n_tail)[cls];
                     ++k;
-                    ++dp.win_n_warps[cls];
                 }
                 ++shares.back().count;
                 done += c;
