@@ -148,6 +148,7 @@ struct TileTemplate {
     int x0, x1, y0, y1;              // owned pixels [x0, x1) x [y0, y1)
     std::vector<Unit> units;         // the tile's units, largest first
     double cost = 0.0;
+    double angle_cost = 1.0;         // of an angle iteration (see angle_cost)
 };
 
 struct GeomTemplate {
@@ -161,6 +162,13 @@ struct GeomTemplate {
 constexpr double kStageCost = 60.0;    // staging a tile, in angle iterations of each warp (30 to 150: within 1 %)
 constexpr int kUnitsPerWarp = 1;       // units per warp from which on a plan uses more CTAs
 constexpr double kUnitOverhead = 3.0;  // per-unit fixed cost, in angle iterations (at 10: 3 % slower at 1024^2)
+// An angle iteration of a plan with radius steps of `delta` pixels, relative to
+// one of fine steps: the further apart the radii of neighbouring lanes, the
+// more distinct cells eight lanes read and the more of them meet in a bank.
+// Measured, in SM cycles: 7.4 to 7.5 up to 0.375 pixels, 8.0 at 0.5, 8.5 at
+// 0.67, 9.1 at 0.75, 9.6 at 1, 10 to 11 from 1.3 to 3.  (Equal weights let the
+// SMs of a batch of 64 uneven instances end up to 30 % after the mean.)
+double angle_cost(double delta) { return 1.0 + 0.48 * std::max(0.0, std::min(delta, 1.25) - 0.33); }
 // Abel tiles of 64 from this many on (forward / adjoint time stage with tiles of
 // 32 and of 64: 10.8 / 10.9 and 12.7 / 11.8 us at 256^2, 128 detectors, 16
 // tiles of 64; 26.7 / 27.0 and 22 / 21 us at 512^2, 256 detectors, 64 tiles)
@@ -331,6 +339,9 @@ pat_status_t build_plan(Plan& P, const pat_geometry_t* geoms, int n_inst, const 
     const int ray_bytes = K_max * (int)sizeof(float4);   // staged beside the tile
     const int64_t cell_budget = std::max<int64_t>(P.band_budget_bytes - ray_bytes, 16 * 1024) / 16;
     const int QL = kWarp / ml;
+    auto unit_cost = [&](const TileTemplate& tt, const Unit& u) {
+        return tt.angle_cost * (double)((u.nq + QL - 1) / QL) + kUnitOverhead;
+    };
 
     for (int i = 0; i < n_inst; ++i) {
         const pat_geometry_t& g = geoms[i];
@@ -552,7 +563,8 @@ pat_status_t build_plan(Plan& P, const pat_geometry_t* geoms, int n_inst, const 
                 const auto& pu = per[x.second][t];
                 tile.units.insert(tile.units.end(), pu.begin(), pu.end());
             }
-            for (const Unit& u : tile.units) tile.cost += (double)(u.nq + QL - 1) / QL + kUnitOverhead;
+            tile.angle_cost = angle_cost(delta);
+            for (const Unit& u : tile.units) tile.cost += unit_cost(tile, u);
         }
     }
 
@@ -576,7 +588,6 @@ pat_status_t build_plan(Plan& P, const pat_geometry_t* geoms, int n_inst, const 
     if (bps < 1) return PAT_ERR_UNSUPPORTED;
     const int n_ctas_target = bps * P.num_sms;
     const int warps_cta = circ_threads / kWarp;
-    auto unit_cost = [&](const Unit& u) { return (double)((u.nq + QL - 1) / QL) + kUnitOverhead; };
     double total_cost = 0.0;
     for (int i = 0; i < n_inst; ++i)
         for (const auto& tt : tmpls[inst_tmpl[i]].tiles) total_cost += tt.cost;
@@ -585,7 +596,7 @@ pat_status_t build_plan(Plan& P, const pat_geometry_t* geoms, int n_inst, const 
     std::vector<std::pair<double, int>> order;
     auto add_lists = [&](const TileTemplate& tt, size_t u0, size_t u1) {
         order.clear();
-        for (size_t u = u0; u < u1; ++u) order.push_back({-unit_cost(tt.units[u]), (int)u});
+        for (size_t u = u0; u < u1; ++u) order.push_back({-unit_cost(tt, tt.units[u]), (int)u});
         std::sort(order.begin(), order.end());
         std::vector<std::vector<Unit>> lists(warps_cta);
         using E = std::pair<double, int>;
@@ -624,7 +635,7 @@ pat_status_t build_plan(Plan& P, const pat_geometry_t* geoms, int n_inst, const 
     for (size_t t = 0; t < tmpls.size(); ++t)
         for (const auto& tt : tmpls[t].tiles) {
             std::vector<double> b(1, 0.0);
-            for (const Unit& u : tt.units) b.push_back(b.back() + unit_cost(u));
+            for (const Unit& u : tt.units) b.push_back(b.back() + unit_cost(tt, u));
             before[t].push_back(std::move(b));
         }
     auto cut = [&](double target, auto&& emit) {
