@@ -52,11 +52,24 @@ std::string tune_key(const pat_geometry_t* geoms, int n, const pat_options_t& op
     return k;
 }
 
+// Mean time of fn over reps calls after warm ones; with a scratch buffer, the
+// time of each call after that was written (which turns everything else out of
+// L2), added up.
 template <typename F>
-float time_ms(cudaStream_t st, int warm, int reps, F&& fn)
+float time_ms(cudaStream_t st, int warm, int reps, F&& fn, void* scratch = nullptr, size_t scratch_bytes = 0)
 {
     for (int i = 0; i < warm; ++i)
         if (fn() != cudaSuccess) return -1.f;
+    if (scratch) {
+        float sum = 0.f;
+        for (int i = 0; i < reps; ++i) {
+            if (cudaMemsetAsync(scratch, i, scratch_bytes, st) != cudaSuccess) return -1.f;
+            const float ms = time_ms(st, 0, 1, fn);
+            if (ms < 0.f) return -1.f;
+            sum += ms;
+        }
+        return sum / (float)reps;
+    }
     cudaEvent_t a, b;
     if (cudaEventCreate(&a) != cudaSuccess) return -1.f;
     if (cudaEventCreate(&b) != cudaSuccess) {
@@ -152,8 +165,10 @@ pat_status_t autotune_plan(Plan** out, const pat_geometry_t* geoms, int n_inst, 
     Plan* best = nullptr;
     float best_ms = 1e30f;
     pat_options_t best_opt = opt;
-    const std::vector<int> ml_c = large ? std::vector<int>{16, 8} : std::vector<int>{32, 16, 8};
-    const std::vector<int> qp_c = large ? std::vector<int>{256} : std::vector<int>{64, 128, 256};
+    // (the untuned shape among them: 32 and 128 on large plans, 155 us at 512^2
+    // where 16 and 256 took 177)
+    const std::vector<int> ml_c = large ? std::vector<int>{32, 16} : std::vector<int>{32, 16, 8};
+    const std::vector<int> qp_c = large ? std::vector<int>{128} : std::vector<int>{64, 128, 256};
     for (int ml : ml_c) {
         for (int qp : qp_c) {
             for (int cols : cols_cands) {
@@ -215,8 +230,17 @@ pat_status_t autotune_plan(Plan** out, const pat_geometry_t* geoms, int n_inst, 
     const std::vector<int> g_c = large ? std::vector<int>{0, 4, 8} : std::vector<int>{0, 1, 2, 4, 8};
     for (int gcount : g_c)
         for (int jb : jb_c) adj_cands.push_back({gcount, jb});
-    // the windowed lists of an automatic plan have no shape to choose and beat
-    // every tuned shape of the per-cell lists (at 512^2: 139 against 188 us)
+    // The windowed lists of an automatic plan are one more candidate.  Where
+    // they are larger than L2 holds they need no comparison (139 against 188 us
+    // at 512^2).  Smaller ones are timed as a program that does other work in
+    // between finds them, with nothing in L2: at 256^2 the gather takes 33 us
+    // over either form when the lists are there, but 45 over the windowed lists
+    // and 35 over the best per-cell shape when they are not (a warp waits for a
+    // block's head and records before it can stage anything).
+    int l2 = 0;
+    if (cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) != cudaSuccess) l2 = 0;
+    void* scratch = nullptr;
+    const size_t scratch_bytes = 2 * (size_t)l2;
     if (opt.adj_mode == 0 && opt.adj_groups == 0 && opt.adj_jblock == 0) {
         pat_options_t o = fwd_opt;
         o.adj_mode = o.adj_groups = 0;
@@ -224,7 +248,19 @@ pat_status_t autotune_plan(Plan** out, const pat_geometry_t* geoms, int n_inst, 
         if (p && p->info.adj_windows) {
             best = p;
             best_opt = o;
-            adj_cands.clear();
+            if (p->info.list_bytes > l2) {
+                adj_cands.clear();
+            } else {
+                if (scratch_bytes > 0 && dev_malloc(&scratch, scratch_bytes) != cudaSuccess) {
+                    cudaGetLastError();
+                    scratch = nullptr;   // (no room: timed as they follow one another)
+                }
+                best_ms = time_ms(st, 2, 5, [&] {
+                    cudaError_t e = launch_abel_adj(p->dp, d_g, st);
+                    return e == cudaSuccess ? launch_adjoint_gather(p->dp, d_f, st) : e;
+                }, scratch, scratch_bytes);
+                if (best_ms < 0.f) best_ms = 1e30f;
+            }
         } else {
             drop(p);
         }
@@ -239,7 +275,7 @@ pat_status_t autotune_plan(Plan** out, const pat_geometry_t* geoms, int n_inst, 
         const float ms = time_ms(st, 2, 5, [&] {
             cudaError_t e = launch_abel_adj(p->dp, d_g, st);
             return e == cudaSuccess ? launch_adjoint_gather(p->dp, d_f, st) : e;
-        });
+        }, scratch, scratch_bytes);
         if (ms > 0.f && ms < best_ms) {
             best_ms = ms;
             drop(best);
@@ -251,6 +287,7 @@ pat_status_t autotune_plan(Plan** out, const pat_geometry_t* geoms, int n_inst, 
     }
     cudaFree(d_f);
     cudaFree(d_g);
+    if (scratch) cudaFree(scratch);
     if (!best) return PAT_ERR_UNSUPPORTED;
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
