@@ -50,11 +50,11 @@ pat_status_t build_plan(Plan& P, const pat_geometry_t* geoms, int n_inst, const 
 void free_plan_memory(Plan& P);
 
 // Windowed adjoint lists (windows_plan.cpp).  windows_fit: whether the staged
-// tables hold every geometry's windows.  build_windows builds them for the
+// tables hold every geometry's windows, and the plan has enough work for them.  build_windows builds them for the
 // plan's instances (inst_tmpl: the geometry template of each) on `st`, fills
 // dp.win_* and the instances' fields (uploaded to d_inst), and gives the
 // device bytes and the most parts a patch is split into.
-bool windows_fit(const pat_geometry_t* geoms, int n_inst);
+bool windows_fit(const pat_geometry_t* geoms, int n_inst, int num_sms);
 pat_status_t build_windows(Plan& P, std::vector<InstDev>& inst, const std::vector<int>& inst_tmpl, int n_tmpl,
                            InstDev* d_inst, int64_t* bytes, int* parts_max, cudaStream_t st);
 

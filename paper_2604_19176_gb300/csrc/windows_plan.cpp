@@ -96,16 +96,27 @@ int32_t win_symmetry(const pat_geometry_t& g, int max_order)
 
 } // namespace
 
-bool windows_fit(const pat_geometry_t* geoms, int n_inst)
+bool windows_fit(const pat_geometry_t* geoms, int n_inst, int num_sms)
 {
-    double windows = 0.0;
+    double windows = 0.0, patches = 0.0, samples = 0.0;   // (about 41 % of a full circle's samples fall on the image)
     for (int i = 0; i < n_inst; ++i) {
         const pat_geometry_t& g = geoms[i];
         // radii across a patch's diagonal (11.31 pixels and the widening), with both ends, the alignment and the padding
         const double delta = g.t_max * g.n / (2.0 * g.n_t);
         if (11.5 / delta + 7.0 > win_slots(4) - 8) return false;
         windows += (double)patches_of(g.n) * patches_of(g.n) * g.n_det;
+        patches += (double)patches_of(g.n) * patches_of(g.n);
+        samples += 0.41 * g.n_det * std::min(g.n_t + 2.0, 2.2 * g.n_t / g.t_max + 2.0) * g.n_angles;
     }
+    // Few patches and little work: a patch is split over many warps, each of
+    // which spends more on beginning and ending than on its entries, and the
+    // per-cell lists are as fast or faster (adjoint over them / over windows:
+    // 18.7 / 20.1 us for 100^2 with 110 detectors, 24.2 / 26.4 for 160^2 with
+    // 100, 26.9 / 32.6 for 128^2 with 256).  From 600 patches (36 / 29 us for
+    // 4 x 140^2 with 48 detectors) or 12 M samples on (48.6 / 41.8 us for 160^2
+    // with 320 detectors, 70.6 / 47.3 for 128^2 with 512) the windows win.
+    const double warps = 20.0 * num_sms;
+    if (patches < warps / 5.0 && samples < 4000.0 * warps) return false;
     return windows * sizeof(int4) <= 4e9;   // (build-time table)
 }
 

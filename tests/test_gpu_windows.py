@@ -16,6 +16,9 @@ from paper_2604_19176_gb300 import Geometry, PatPlan, inputs
 pytestmark = pytest.mark.gpu
 
 TOL = 1e-5   # the stated FP32 parity bound of A and A^T
+# Plans of few patches and little work keep the per-cell lists: a large image with one detector brings a plan of small
+# geometries above that line.
+LARGE = Geometry(248, 1, 0.9, 1.0, 20, 2.0, 31)
 
 
 def _adjoint_error(plan, geoms, dev, seed):
@@ -58,9 +61,10 @@ def _adjoint_error(plan, geoms, dev, seed):
     Geometry(248, 90, 0.0, math.pi, 1400, 2.0, 96),          # 6 radii per pixel
 ])
 def test_windowed_adjoint(cuda_dev, g):
-    plan = PatPlan(g, device=cuda_dev)
+    geoms = [g, LARGE] if g.n < 200 else [g]
+    plan = PatPlan(geoms, device=cuda_dev)
     assert plan.info()["adj_windows"] == 1
-    assert _adjoint_error(plan, [g], cuda_dev, 5) <= TOL
+    assert _adjoint_error(plan, geoms, cuda_dev, 5) <= TOL
     # and the transpose of the forward operator
     gen = torch.Generator(device=cuda_dev).manual_seed(6)
     f = torch.randn(plan.image_shape(), generator=gen, device=cuda_dev)
@@ -92,11 +96,14 @@ def test_identical_instances_share_lists(cuda_dev, counts):
         assert not out[:fo[i]].any() and not out[fo[i + 1]:].any()
 
 
-def test_fine_radius_steps_keep_the_per_cell_lists(cuda_dev):
-    g = Geometry(8, 3, 0.0, math.pi, 420, 2.0, 24)   # 52 radii per pixel: more than a block stages
-    plan = PatPlan(g, device=cuda_dev)
+@pytest.mark.parametrize("geoms", [
+    [Geometry(8, 3, 0.0, math.pi, 420, 2.0, 24), LARGE],   # 52 radii per pixel: more than a block stages
+    [Geometry(64, 40, 0.0, math.pi, 128, 2.0, 128)],       # few patches, little work
+])
+def test_plans_that_keep_the_per_cell_lists(cuda_dev, geoms):
+    plan = PatPlan(geoms, device=cuda_dev)
     assert plan.info()["adj_windows"] == 0 and plan.info()["adj_mode"] == 4
-    assert _adjoint_error(plan, [g], cuda_dev, 31) <= TOL
+    assert _adjoint_error(plan, geoms, cuda_dev, 31) <= TOL
 
 
 @pytest.mark.parametrize("g,count", [
