@@ -658,7 +658,7 @@ def main():
         plan.tv_step(f_bufs[k & 1], f_bufs[(k + 1) & 1], g_meas, tau, LAM, EPS, nonneg=True)
         it[0] = k + 1
 
-    launches_per_step = 5  # circular means, Abel forward+residual, Abel adjoint, adjoint gather, TV update
+    launches_per_step = 4  # circular means, fused time stage, adjoint gather, TV update
     for _ in range(max(3, args.warmup)):
         step()
     torch.cuda.synchronize()

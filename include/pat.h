@@ -106,7 +106,8 @@ typedef struct {
     int32_t adj_groups;  /* detector groups of the adjoint gather, 1..16; 0 = auto           */
     int32_t adj_mode;    /* adjoint gather: 0 = auto (windowed code lists where adj_groups    */
                          /*   and adj_jblock are 0 too, the radii that cross 8 pixels fit the */
-                         /*   staged tables and the codes the list budget; else 4 if it fits  */
+                         /*   staged tables, the codes the list budget, and the plan has 600  */
+                         /*   patches of 8 x 8 pixels or some 12 M samples; else 4 if it fits */
                          /*   the budget, else 1, else 3, else 2);                            */
                          /*   1 = per-cell sample code lists built at                         */
                          /*   creation (device memory ~4 B per sample); 2 = enumerate on      */
@@ -195,8 +196,9 @@ pat_status_t pat_forward(pat_plan_t plan, const void* d_f, float* d_g, void* str
  * pat_adjoint — f = A^T g for every instance: the exact transpose of the
  * discrete A above, the operator whose application gives the data-term
  * gradient of Eq. (4) and Eq. (5) (Sec. 2.2).  Evaluated as a gather over
- * pixels (each output element is summed by one thread in a fixed order; no
- * atomics), so results are deterministic.
+ * pixels in a fixed order: every part of a pixel's sum is made by one warp,
+ * and the parts are added in their order by whichever warp is last (no
+ * floating-point atomics), so results are deterministic.
  *   d_g: device, packed FP32 data (read only).
  *   d_f: device, packed images in the plan's image dtype, overwritten.
  */
@@ -309,7 +311,7 @@ pat_status_t pat_pdhg_step(pat_plan_t plan, float* d_f, float* d_fbar, float* d_
  * affected (the circular-mean kernel keeps no state across calls; its work is
  * scheduled statically).  The status word stays set until this call reports
  * and clears it (it also re-arms the adjoint kernels' work queues, which no
- * bounded wait can leave armed).
+ * bounded wait can leave armed: the gathers wait for nothing).
  */
 pat_status_t pat_plan_sync_status(pat_plan_t plan, void* stream);
 

@@ -18,8 +18,9 @@ __device__ __forceinline__ float ld_img(const __nv_bfloat16* p) { return __bfloa
 // Sample coordinates in split form (the coordinate conventions of
 // pat_internal.h).  cell_rel: cell of radius index mf along direction
 // component hi, relative to the detector's integer part, from the detector's
-// fraction f0.  cell_frac: the sample's fraction inside that cell.  Both
-// the forward and the adjoint gathers call exactly these.
+// fraction f0.  cell_frac: the sample's fraction inside that cell.  The
+// adjoint's per-cell forms call exactly these, and the forward evaluates the
+// same sequence in pairs (the windowed lists are in fixed point, windows.cu).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ float cell_rel(float mf, float hi, float f0)
 {

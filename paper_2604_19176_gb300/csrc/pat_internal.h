@@ -23,10 +23,12 @@
 // fraction at any N (the cell decision itself may differ from the exact one
 // only for samples within ~N * 2^-24 of a grid line, where both cells give
 // the same interpolated value to that order).  The forward gather and the
-// adjoint gather evaluate exactly these expressions (explicit __fmaf_rn /
-// __fadd_rn, no contraction freedom), so both kernels see every sample in
-// the same cell with the same bilinear weights: the adjoint is the transpose
-// of the forward matrix.
+// per-cell forms of the adjoint evaluate exactly these expressions (explicit
+// __fmaf_rn / __fadd_rn, no contraction freedom), so they see every sample in
+// the same cell with the same bilinear weights.  The windowed adjoint (the
+// default) holds positions in 32-bit fixed point, at least as close to the
+// exact ones (windows.cu); its matrix is the forward's transpose to the
+// rounding of either.
 #pragma once
 
 #include <cstddef>
@@ -39,8 +41,9 @@ constexpr int kPatchW = 8;        // adjoint: one warp owns an 8 x 4 patch of ce
 constexpr int kPatchH = 4;
 // Work queues live kQueueStride ints apart (one 128-byte line each, so that
 // queues taken by different CTAs do not serialise on one L2 line): queue 0 is
-// the adjoint cell kernel's (the list kernel's schedule is static).  Each
-// queue is two ints: the next item and the count of finished participants.
+// the adjoint cell kernel's, queue 1 the last shares' of the list kernels (one
+// of which a plan uses).  Each queue is two ints: the next item and the count
+// of finished participants.
 constexpr int kQueueStride = 32;
 
 // Per-instance descriptor (device resident, read by every kernel).

@@ -36,7 +36,9 @@
 // at a barrier per block, left the warps waiting for the longest list more
 // than half of the time: 61 us at 256^2).  The blocks of all patches and
 // instances form one sequence, cut into equal-cost shares, one per resident
-// warp, so a patch is split over a few warps where there are few patches.  A
+// warp, so a patch is split over a few warps where there are few patches; on
+// large plans (TAIL) the end of the sequence makes smaller shares, which the
+// warps take from a queue as they run out (kTailFrom in windows_plan.cpp).  A
 // warp adds its cells' corner sums into 9 x 9 pixel sums and writes those (81
 // values instead of 256), which the combining kernels add (adj_pixel).
 //
@@ -57,8 +59,9 @@
 // wavefronts and 79 M warp instructions, 70 % of the L1 data path's peak.
 // Gather and combine, per-cell run-pair lists -> windowed lists: 49 -> 32 us
 // at 256^2 (128 detectors, half ring), 328 -> 139 us at 512^2, 595 -> 330 us
-// at 760^2 (256 detectors, 270 degrees), 3.53 -> 1.98 ms for 64 uneven
-// instances, 13.4 -> 5.3 ms for 8 x 1024^2.
+// at 760^2 (256 detectors, 270 degrees), 3.53 -> 1.75 ms for 64 uneven
+// instances, 13.4 -> 4.8 ms for 8 x 1024^2 (90 % of the L1 data path's peak
+// in the uneven batch; two fifths of the wavefronts are bank conflicts).
 #include <algorithm>
 
 #include "device_common.cuh"
