@@ -101,14 +101,19 @@ cudaError_t launch_adj_seg(const DevPlan& dp, int inst_idx, int n, bool pairs, i
                            const int64_t* pbase, uint32_t* out, cudaStream_t st);
 
 // Windowed lists (windows.cu): the gather, and the steps of list building
-// (windows of every detector and patch; their cut into blocks, counting when
-// blocks == nullptr; staging records; codes, counting when codes == nullptr).
+// (windows of every detector and patch; the samples that need a position of
+// their own, the first `cap` of them kept; the cut of both into blocks,
+// counting when blocks == nullptr; staging records; codes, counting when
+// codes == nullptr).
 cudaError_t launch_adj_win(const DevPlan& dp, cudaStream_t st);
 int adj_win_blocks_per_sm(int nb);
 cudaError_t launch_win_windows(const DevPlan& dp, int inst_idx, int n_det, double delta, int patches, int4* win,
                                cudaStream_t st);
+cudaError_t launch_win_own(const DevPlan& dp, int inst_idx, int n_det, int patches, int patch0, const int4* win,
+                           WinOwn* own, uint32_t cap, uint32_t* count, cudaStream_t st);
 cudaError_t launch_win_part(const DevPlan& dp, int inst_idx, int patches, int max_rays, int max_slots, int max_longest,
-                            const int4* win, int4* cnt, WinBlock* blocks, WinSub* subs, int32_t* err, cudaStream_t st);
+                            const int4* win, const WinOwn* own, int n_own, int4* cnt, WinBlock* blocks, WinSub* subs,
+                            int32_t* err, cudaStream_t st);
 cudaError_t launch_win_recs(const DevPlan& dp, int inst_idx, int n_blocks, const WinBlock* blocks, const WinSub* subs,
                             uint2* rayrec, uint32_t* slotrec, cudaStream_t st);
 cudaError_t launch_win_lists(const DevPlan& dp, int inst_idx, int n_blocks, WinBlock* blocks, const WinSub* subs,

@@ -26,9 +26,10 @@
 // per-cell forms of the adjoint evaluate exactly these expressions (explicit
 // __fmaf_rn / __fadd_rn, no contraction freedom), so they see every sample in
 // the same cell with the same bilinear weights.  The windowed adjoint (the
-// default) holds positions in 32-bit fixed point, at least as close to the
-// exact ones (windows.cu); its matrix is the forward's transpose to the
-// rounding of either.
+// default) holds positions in 32-bit fixed point, closer to the exact ones up
+// to some 30 radii per pixel (windows.cu), and gives every sample one cell
+// (win_position.h); its matrix is the forward's transpose to the rounding of
+// either.
 #pragma once
 
 #include <cstddef>
@@ -191,10 +192,17 @@ struct WinBlock {
 };
 
 // Rays q0 .. q0 + nq - 1 (mod K) and radii m0 .. m0 + nm - 1 of detector j,
-// staged from ray slot ray0 and radius slot slot0 (list building only).
+// staged from ray slot ray0 and radius slot slot0 with positions anchored at
+// radius mc (list building only).  own: only the sample (q0, mc) of them, one
+// that the patch's window of detector j cannot hold (win_position.h).
 struct WinSub {
-    int32_t j, q0, nq, m0, nm;
+    int32_t j, q0, nq, m0, nm, mc, own;
     uint16_t ray0, slot0;
+};
+
+// Such a sample: its patch, detector, angle and radius.
+struct WinOwn {
+    int32_t patch, j, q, m;
 };
 
 // Symmetry of a geometry: maps of the square that take its detectors to its

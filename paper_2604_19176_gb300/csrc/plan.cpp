@@ -16,6 +16,7 @@
 
 #include "kernels.h"
 #include "plan.h"
+#include "win_position.h"
 
 namespace patgpu {
 
@@ -220,21 +221,6 @@ void choose_tile(int n, int64_t cells, int want_w, int want_h, int& tw, int& th)
     }
 }
 
-// x as whole + frac / 2^64
-struct Fixed {
-    int32_t whole;
-    uint64_t frac;
-};
-Fixed fixed_of(double x)
-{
-    double w = std::floor(x), f = x - w;
-    if (f >= 1.0) {   // (x a rounding error below a whole number)
-        w += 1.0;
-        f = 0.0;
-    }
-    return {(int32_t)w, (uint64_t)(f * 18446744073709551616.0)};
-}
-
 } // namespace
 
 static_assert(sizeof(InstDev) % 8 == 0, "InstDev layout");
@@ -384,16 +370,8 @@ pat_status_t build_plan(Plan& P, const pat_geometry_t* geoms, int n_inst, const 
             const double ui = std::floor((double)uf), vi = std::floor((double)vf);
             det4.push_back(make_float4((float)ui, (float)vi, (float)(ue - ui), (float)(ve - vi)));
             if (win_wanted) {
-                const Fixed u = fixed_of(ue), v = fixed_of(ve);
-                // (32 fraction bits, rounded; a carry goes to the integer part)
-                auto hi32 = [](const Fixed& f, int32_t& whole) {
-                    const uint64_t r = (f.frac >> 32) + ((f.frac >> 31) & 1u);
-                    whole = f.whole + (int32_t)(r >> 32);
-                    return (int32_t)(uint32_t)r;
-                };
-                int32_t iu = 0, iv = 0;
-                const int32_t fu = hi32(u, iu), fv = hi32(v, iv);
-                win_det.push_back(make_int4(fu, fv, iu, iv));
+                const int64_t u = win_detector(ue), v = win_detector(ve);
+                win_det.push_back(make_int4((int32_t)(uint32_t)u, (int32_t)(uint32_t)v, win_cell(u), win_cell(v)));
             }
         }
         // M / Mbar row pitch and the adjoint list code q << (jb + mb) | j << mb | m

@@ -16,12 +16,15 @@
 //     u = X + offset * D  (mod 2^32),   a = u / 2^32 .
 // The cell is known (it is the lane's), so the integer part is never needed.
 // X is formed at the centre radius of the window from 64-bit tables; the step
-// is rounded to 2^-30 pixel, so u is within 2^-31 x (radii from the centre, at
-// most half a window, ~32) + 2^-32 of the exact position: better than the
-// 3 x 2^-25 of the FP32 split form.  The lists are built with the same integer
-// arithmetic, integer part included, so no sample can wrap around its cell.
-// The fraction is read as the 23-bit mantissa of 1 + a, centred in its
-// truncation interval.
+// is rounded to 2^-30 pixel, so u is within 2^-31 x (radii from the centre) +
+// 2^-32 of the exact position: 6e-9 pixel at two radii per pixel (13 from the
+// centre), 1.3e-7 at the finest radii that a patch's window may have (some 48
+// per pixel, 275 from the centre); the FP32 split form is within 3 x 2^-25 =
+// 9e-8.  Which cell of which patch lists a sample is decided by its position
+// formed at its own radius, the same in every patch; the few samples whose
+// staged position lies in another cell get a staged ray of their own
+// (win_position.h).  The fraction is read as the 23-bit mantissa of 1 + a,
+// centred in its truncation interval.
 //
 // Lists.  Two samples of one ray at consecutive radii in one cell make a pair
 // entry; others are single.  Half a patch (8 x 4 cells, lane = cell) has, per
@@ -66,6 +69,7 @@
 
 #include "device_common.cuh"
 #include "kernels.h"
+#include "win_position.h"
 
 namespace patgpu {
 
@@ -492,56 +496,80 @@ __device__ __forceinline__ void patch_cells(const InstDev& in, int p, int& x0, i
 
 } // namespace
 
-// win[j * patches + p] = (q0, nq, m0, nm | near << 16): every sample of detector j that
-// lands in patch p has its ray in q0 .. q0 + nq - 1 (mod K) and its radius in
-// m0 .. m0 + nm - 1.  The patch is widened by 0.02 pixel (the positions' error
-// is below 1e-3), its distance range gives the radii and its corners' angles
-// the rays; a detector within half a pixel sees the whole circle.
+// win[j * patches + p] = (q0, nq, m0, nm | near << 16): the range of detector j
+// and patch p (win_range).
 __global__ void k_win_windows(DevPlan dp, int inst_idx, double delta, int patches, int4* __restrict__ win)
 {
     const InstDev in = dp.inst[inst_idx];
     const int p = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
     if (p >= patches) return;
+    int x0, y0, x1, y1;
+    patch_cells(in, p, x0, y0, x1, y1);
     for (int jj = j; jj < in.win_ndet; jj += gridDim.y) {
         const int4 d = dp.win_det[in.det_off + jj];
         const double U = (double)d.z + (double)(uint32_t)d.x * (1.0 / 4294967296.0);
         const double V = (double)d.w + (double)(uint32_t)d.y * (1.0 / 4294967296.0);
+        const WinRange r =
+            win_range(U, V, x0 - in.c0, y0 - in.c0, x1 - in.c0, y1 - in.c0, in.K, in.n_r, in.m_pitch, delta);
+        win[(size_t)jj * patches + p] = make_int4(r.q0, r.nq, r.m0, r.nm | r.near << 16);
+    }
+}
+
+namespace {
+
+// Fixed-point detector and direction of a sample's ray.
+struct RayFixed {
+    int4 det;
+    uint4 dir;
+    int2 whole;
+    __device__ __forceinline__ int64_t u(int m) const
+    {
+        return win_position((int64_t)det.z * 4294967296ll + (int64_t)(uint32_t)det.x, whole.x, dir.x, dir.z, m);
+    }
+    __device__ __forceinline__ int64_t v(int m) const
+    {
+        return win_position((int64_t)det.w * 4294967296ll + (int64_t)(uint32_t)det.y, whole.y, dir.y, dir.w, m);
+    }
+};
+__device__ __forceinline__ RayFixed ray_fixed(const DevPlan& dp, const InstDev& in, int j, int q)
+{
+    return {__ldg(dp.win_det + in.det_off + j), __ldg(dp.win_dirs + in.win_ray_off + q),
+            __ldg(dp.win_dirs_int + in.win_ray_off + q)};
+}
+
+} // namespace
+
+// The samples of every window that land in its patch but whose staged position
+// lands in another cell: (patch0 + patch, j, q, m) into own[], the first `cap`
+// of them in no order; *count counts all.  A warp per window, lane = ray.
+__global__ void __launch_bounds__(256) k_win_own(DevPlan dp, int inst_idx, int patches, int patch0,
+                                                 const int4* __restrict__ win, WinOwn* __restrict__ own, uint32_t cap,
+                                                 uint32_t* __restrict__ count)
+{
+    const InstDev in = dp.inst[inst_idx];
+    const int lane = threadIdx.x & 31;
+    const int64_t n_win = (int64_t)patches * in.win_ndet;
+    for (int64_t w = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); w < n_win; w += (int64_t)gridDim.x * 8) {
+        const int4 wv = win[w];
+        const int nm = wv.w & 0xffff, m0 = wv.z;
+        if (wv.y <= 0 || nm <= 0) continue;
+        const int j = (int)(w / patches), p = (int)(w % patches), mc = win_anchor(m0, nm);
         int x0, y0, x1, y1;
         patch_cells(in, p, x0, y0, x1, y1);
-        const double eps = 0.02;
-        const double ax = x0 - in.c0 - eps - U, bx = x1 - in.c0 + eps - U;
-        const double ay = y0 - in.c0 - eps - V, by = y1 - in.c0 + eps - V;
-        const double nx = fmax(0.0, fmax(ax, -bx)), ny = fmax(0.0, fmax(ay, -by));
-        const double fx = fmax(fabs(ax), fabs(bx)), fy = fmax(fabs(ay), fabs(by));
-        const double rmin = sqrt(nx * nx + ny * ny), rmax = sqrt(fx * fx + fy * fy);
-        int m0 = (int)fmin(1e6, ceil(rmin / delta - 1e-6)), m1 = (int)fmin((double)(in.n_r - 1), floor(rmax / delta + 1e-6));
-        int4 o = make_int4(0, 0, 0, 0);
-        if (m0 <= m1) {
-            int q0 = 0, nq = in.K;
-            if (rmin > 0.5) {
-                const double cx = 0.5 * (ax + bx), cy = 0.5 * (ay + by);
-                double lo = 0.0, hi = 0.0;
-                const double px[4] = {ax, bx, ax, bx}, py[4] = {ay, ay, by, by};
-                for (int i = 0; i < 4; ++i) {
-                    const double a = atan2(cx * py[i] - cy * px[i], cx * px[i] + cy * py[i]);
-                    lo = fmin(lo, a);
-                    hi = fmax(hi, a);
-                }
-                const double per = in.K / 6.283185307179586476925, pc = atan2(cy, cx);
-                const int qa = (int)ceil((pc + lo) * per - 1e-3), qb = (int)floor((pc + hi) * per + 1e-3);
-                nq = min(qb - qa + 1, in.K);
-                q0 = nq == in.K ? 0 : ((qa % in.K) + in.K) % in.K;
-            }
-            if (nq > 0) {
-                m0 &= ~3;   // (16-byte reads of Mbar)
-                const int nmp = pad_to(m1 - m0 + 1, 8);
-                if (m0 + nmp > in.m_pitch) m0 = max(0, in.m_pitch - nmp);   // (padded radii stay inside the row)
-                // rays through the nearest cell: what the longest list of the patch gets from this window
-                const double near = fmin(32767.0, ceil(1.3 * in.K / (6.283185307179586476925 * fmax(rmin, 0.7))));
-                o = make_int4(q0, nq, m0, (m1 - m0 + 1) | (int)near << 16);
+        for (int i = lane; i < wv.y; i += kWarp) {
+            int q = wv.x + i;
+            if (q >= in.K) q -= in.K;
+            const RayFixed r = ray_fixed(dp, in, j, q);
+            const int64_t uc = r.u(mc), vc = r.v(mc);
+            const int64_t su = win_step(r.whole.x, r.dir.x), sv = win_step(r.whole.y, r.dir.y);
+            for (int m = m0; m < m0 + nm; ++m) {
+                const int cx = win_cell(r.u(m)), cy = win_cell(r.v(m));
+                if (win_cell(win_staged(uc, su, m, mc)) == cx && win_cell(win_staged(vc, sv, m, mc)) == cy) continue;
+                if (cx + in.c0 < x0 || cx + in.c0 >= x1 || cy + in.c0 < y0 || cy + in.c0 >= y1) continue;
+                const uint32_t at = atomicAdd(count, 1u);
+                if (at < cap) own[at] = {patch0 + p, j, q, m};
             }
         }
-        win[(size_t)jj * patches + p] = o;
     }
 }
 
@@ -549,11 +577,13 @@ __global__ void k_win_windows(DevPlan dp, int inst_idx, double delta, int patche
 // tables (max_rays rays, max_slots radii) and whose longest list stays near
 // max_longest entries (the warps are the unit of scheduling, and the cells
 // next to a detector see every one of its rays); a window of more rays becomes
-// several.  With blocks == nullptr counts (blocks, sub-windows, ray and slot
+// several.  The patch's samples of own[] (n_own, ascending) follow, one
+// sub-window each.  With blocks == nullptr counts (blocks, sub-windows, ray and slot
 // groups) per patch into cnt; else writes them from the offsets in cnt.
 __global__ void k_win_part(DevPlan dp, int inst_idx, int patches, int max_rays, int max_slots, int max_longest,
-                           const int4* __restrict__ win, int4* __restrict__ cnt, WinBlock* __restrict__ blocks,
-                           WinSub* __restrict__ subs, int32_t* __restrict__ err)
+                           const int4* __restrict__ win, const WinOwn* __restrict__ own, int n_own,
+                           int4* __restrict__ cnt, WinBlock* __restrict__ blocks, WinSub* __restrict__ subs,
+                           int32_t* __restrict__ err)
 {
     const InstDev in = dp.inst[inst_idx];
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
@@ -580,43 +610,47 @@ __global__ void k_win_part(DevPlan dp, int inst_idx, int patches, int max_rays, 
         sg += (slots - 8) / 8;
         open = false;
     };
+    // rays q0 .. q0 + n - 1 and radii m0 .. m0 + nm - 1 of detector j, anchored at mc; len: their part of the longest list
+    // (an odd number of fours: the next window's rays then start in the other half of the eight
+    // 16-byte bank groups; shared-memory conflicts of the gather, 144 -> 138 us at 512^2)
+    auto add = [&](int j, int q0, int n, int m0, int nm, int mc, int len, int own_sample) {
+        const int n4 = min(pad_to(n, 4) | 4, max_rays), nmp = pad_to(nm, 8);
+        if (open && (rays + n4 > max_rays || slots + nmp > max_slots || longest + len > max_longest)) close();
+        if (!open) {
+            open = true;
+            rays = longest = 0;
+            slots = 8;
+            sub_first = ns;
+        }
+        if (subs) subs[base.y + ns] = {j, q0, n, m0, nm, mc, own_sample, (uint16_t)rays, (uint16_t)slots};
+        rays += n4;
+        slots += nmp;
+        longest += len;
+        ++ns;
+    };
     for (int j = 0; j < in.win_ndet; ++j) {
         const int4 wv = win[(size_t)j * patches + p];
         const int nm = wv.w & 0xffff, near = wv.w >> 16;
         if (wv.y <= 0 || nm <= 0) continue;
-        const int nmp = pad_to(nm, 8);
-        if (8 + nmp > max_slots) {
+        if (8 + pad_to(nm, 8) > max_slots) {
             if (!blocks) atomicExch(err, 1);
             return;
         }
         const int chunk = near > max_longest ? min(max_rays, max_longest) : max_rays;
-        // (an odd number of fours: the next window's rays then start in the other half of the eight
-        // 16-byte bank groups; shared-memory conflicts of the gather, 144 -> 138 us at 512^2)
         for (int qd = 0; qd < wv.y; qd += chunk) {
-            const int n = min(chunk, wv.y - qd), n4 = min(pad_to(n, 4) | 4, max_rays), len = min(n, near);
-            if (open && (rays + n4 > max_rays || slots + nmp > max_slots || longest + len > max_longest)) close();
-            if (!open) {
-                open = true;
-                rays = longest = 0;
-                slots = 8;
-                sub_first = ns;
-            }
-            if (subs) {
-                WinSub s;
-                s.j = j;
-                s.q0 = (wv.x + qd) % in.K;
-                s.nq = n;
-                s.m0 = wv.z;
-                s.nm = nm;
-                s.ray0 = (uint16_t)rays;
-                s.slot0 = (uint16_t)slots;
-                subs[base.y + ns] = s;
-            }
-            rays += n4;
-            slots += nmp;
-            longest += len;
-            ++ns;
+            const int n = min(chunk, wv.y - qd);
+            add(j, (wv.x + qd) % in.K, n, wv.z, nm, win_anchor(wv.z, nm), min(n, near), 0);
         }
+    }
+    int o = 0;   // the patch's first
+    for (int hi = n_own; o < hi;) {
+        const int mid = (o + hi) / 2;
+        if (own[mid].patch < p) o = mid + 1;
+        else hi = mid;
+    }
+    for (; o < n_own && own[o].patch == p; ++o) {
+        const int m = own[o].m, m0 = max(0, min(m & ~3, in.m_pitch - 8));   // (eight radii, 16-byte reads)
+        add(own[o].j, own[o].q, 1, m0, m - m0 + 1, m, 1, 1);
     }
     close();
     if (!blocks) cnt[p] = make_int4(nb, ns, rg, sg);
@@ -632,11 +666,10 @@ __global__ void k_win_recs(DevPlan dp, int inst_idx, const WinBlock* __restrict_
     const WinBlock b = blocks[blockIdx.x];
     for (uint32_t i = 0; i < b.n_sub; ++i) {
         const WinSub s = subs[b.sub0 + i];
-        const int mc = s.m0 + s.nm / 2;
         for (int g = threadIdx.x; 4 * g < s.nq; g += blockDim.x)
             rayrec[b.ray_rec + s.ray0 / 4 + g] =
-                make_uint2((uint32_t)s.j | (uint32_t)mc << 14,
-                           (uint32_t)((s.q0 + 4 * g) % in.K) | (uint32_t)(s.slot0 + mc - s.m0) << 16);
+                make_uint2((uint32_t)s.j | (uint32_t)s.mc << 14,
+                           (uint32_t)((s.q0 + 4 * g) % in.K) | (uint32_t)(s.slot0 + s.mc - s.m0) << 16);
         for (int g = threadIdx.x; 8 * g < s.nm; g += blockDim.x)
             slotrec[b.slot_rec + (s.slot0 - 8) / 8 + g] = (uint32_t)s.j * (uint32_t)in.m_pitch + (uint32_t)(s.m0 + 8 * g);
     }
@@ -649,13 +682,18 @@ namespace {
 constexpr float kWinRcell = 0.70710678f + 0.004f, kWinSlabEps = 0.01f, kWinAngMargin = 1.0e-5f;
 
 // Calls hit(rel, m) for the samples of sub-window s (ray q0 + rel, radius m)
-// that land in centred cell (cxi, cyi), rays ascending from the cell's first,
-// radii ascending.  A sample's cell is the integer part of exactly the fixed
-// point position whose fraction k_adj_win uses.
+// that land in centred cell (cxi, cyi) and whose staged position, the one whose
+// fraction k_adj_win uses, lands there too, rays ascending from the cell's
+// first, radii ascending.
 template <typename Hit>
 __device__ __forceinline__ void enumerate_window(const DevPlan& dp, const InstDev& in, const WinSub& s, int cxi,
                                                  int cyi, Hit&& hit)
 {
+    if (s.own) {
+        const RayFixed r = ray_fixed(dp, in, s.j, s.q0);
+        if (win_cell(r.u(s.mc)) == cxi && win_cell(r.v(s.mc)) == cyi) hit(0, s.mc);
+        return;
+    }
     const float cxf = (float)cxi, cyf = (float)cyi;
     const float4 d = __ldg(dp.det + in.det_off + s.j);
     const float U = d.x + d.z, V = d.y + d.w;
@@ -676,10 +714,6 @@ __device__ __forceinline__ void enumerate_window(const DevPlan& dp, const InstDe
     const float ax0 = (cxf - kWinSlabEps) - U, ax1 = (cxf + 1.f + kWinSlabEps) - U;
     const float ay0 = (cyf - kWinSlabEps) - V, ay1 = (cyf + 1.f + kWinSlabEps) - V;
     const float2* rtrig = dp.rtrig + in.ray_off;
-    const int4 di = dp.win_det[in.det_off + s.j];
-    const long long u0 = ((long long)di.z << 32) + (long long)(uint32_t)di.x;
-    const long long v0 = ((long long)di.w << 32) + (long long)(uint32_t)di.y;
-    const int mc = s.m0 + s.nm / 2;
     for (int i = 0; i < qn; ++i) {
         int q = qlo + i;
         if (q >= K) q -= K;
@@ -693,14 +727,13 @@ __device__ __forceinline__ void enumerate_window(const DevPlan& dp, const InstDe
         const float hi = fminf(fmaxf(tx0, tx1), fmaxf(ty0, ty1));
         const int m0 = max(max(mlo, (int)ceilf(lo)), s.m0), m1 = min(min(mhi, (int)floorf(hi)), s.m0 + s.nm - 1);
         if (m0 > m1) continue;
-        const uint4 r = __ldg(dp.win_dirs + in.win_ray_off + q);
-        const int2 ri2 = __ldg(dp.win_dirs_int + in.win_ray_off + q);
-        const long long xc = u0 + (((long long)mc * ri2.x) << 32) + (long long)mc * (long long)r.x + __umulhi((uint32_t)mc, r.z);
-        const long long yc = v0 + (((long long)mc * ri2.y) << 32) + (long long)mc * (long long)r.y + __umulhi((uint32_t)mc, r.w);
-        const long long sx = ((long long)ri2.x << 32) + (long long)(((unsigned long long)r.x + 2ull) & ~3ull);
-        const long long sy = ((long long)ri2.y << 32) + (long long)(((unsigned long long)r.y + 2ull) & ~3ull);
+        const RayFixed r = ray_fixed(dp, in, s.j, q);
+        const int64_t uc = r.u(s.mc), vc = r.v(s.mc);
+        const int64_t su = win_step(r.whole.x, r.dir.x), sv = win_step(r.whole.y, r.dir.y);
         for (int m = m0; m <= m1; ++m)
-            if ((int)((xc + (m - mc) * sx) >> 32) == cxi && (int)((yc + (m - mc) * sy) >> 32) == cyi) hit(rel, m);
+            if (win_cell(win_staged(uc, su, m, s.mc)) == cxi && win_cell(win_staged(vc, sv, m, s.mc)) == cyi &&
+                win_cell(r.u(m)) == cxi && win_cell(r.v(m)) == cyi)
+                hit(rel, m);
     }
 }
 
@@ -857,11 +890,20 @@ cudaError_t launch_win_windows(const DevPlan& dp, int inst_idx, int n_det, doubl
     return cudaGetLastError();
 }
 
-cudaError_t launch_win_part(const DevPlan& dp, int inst_idx, int patches, int max_rays, int max_slots, int max_longest,
-                            const int4* win, int4* cnt, WinBlock* blocks, WinSub* subs, int32_t* err, cudaStream_t st)
+cudaError_t launch_win_own(const DevPlan& dp, int inst_idx, int n_det, int patches, int patch0, const int4* win,
+                           WinOwn* own, uint32_t cap, uint32_t* count, cudaStream_t st)
 {
-    k_win_part<<<(patches + 63) / 64, 64, 0, st>>>(dp, inst_idx, patches, max_rays, max_slots, max_longest, win, cnt,
-                                                   blocks, subs, err);
+    const int64_t blocks = ((int64_t)n_det * patches + 7) / 8;
+    k_win_own<<<(unsigned)std::min<int64_t>(blocks, 1 << 20), 256, 0, st>>>(dp, inst_idx, patches, patch0, win, own, cap, count);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_win_part(const DevPlan& dp, int inst_idx, int patches, int max_rays, int max_slots, int max_longest,
+                            const int4* win, const WinOwn* own, int n_own, int4* cnt, WinBlock* blocks, WinSub* subs,
+                            int32_t* err, cudaStream_t st)
+{
+    k_win_part<<<(patches + 63) / 64, 64, 0, st>>>(dp, inst_idx, patches, max_rays, max_slots, max_longest, win, own,
+                                                   n_own, cnt, blocks, subs, err);
     return cudaGetLastError();
 }
 

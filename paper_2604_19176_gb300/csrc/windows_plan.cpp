@@ -4,6 +4,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <tuple>
 #include <vector>
 
 #include <cuda_runtime.h>
@@ -60,6 +61,9 @@ double block_cost(const WinBlock& b, int nb)
 constexpr double kTailFrom = 1e5, kTailPart = 0.25, kTailShare = 0.05;
 constexpr double kFlushCost = 100.0;   // end of a patch, per instance
 
+// Samples with a position of their own that the first pass has room for (5 x
+// 10^8 samples at 8 radii per pixel have some ten).
+constexpr uint32_t kOwnFirst = 1 << 12;
 constexpr double kPatchRays = 11.0;   // rays of a detector that an 8 x 8 patch sees, about
 constexpr int kMinRays = 96;
 
@@ -182,21 +186,66 @@ pat_status_t build_windows(Plan& P, std::vector<InstDev>& inst, const std::vecto
     }
     DevBuf tmp(st);
     const size_t o_cnt = align256(sizeof(int4) * win_off[n_tmpl]);
-    const size_t o_misc = o_cnt + align256(sizeof(int4) * patch_off[n_tmpl]);
+    const size_t o_own = o_cnt + align256(sizeof(int4) * patch_off[n_tmpl]);
+    const size_t o_misc = o_own + align256(sizeof(WinOwn) * kOwnFirst);
     if (!tmp.alloc(o_misc + 256)) return PAT_ERR_OOM;
     unsigned char* tb = static_cast<unsigned char*>(tmp.p);
     int4* d_win = reinterpret_cast<int4*>(tb);
     int4* d_cnt = reinterpret_cast<int4*>(tb + o_cnt);
     int32_t* d_err = reinterpret_cast<int32_t*>(tb + o_misc);
     if (cudaMemsetAsync(d_err, 0, sizeof(int32_t), st) != cudaSuccess) return PAT_ERR_CUDA;
+    if (patch_off[n_tmpl] > INT32_MAX) return PAT_ERR_UNSUPPORTED;
     for (int t = 0; t < n_tmpl; ++t) {
         const int i = rep[t], np = (int)(patch_off[t + 1] - patch_off[t]);
         const double delta = P.geoms[i].t_max * P.geoms[i].n / (2.0 * P.geoms[i].n_t);
-        if (launch_win_windows(dp, i, inst[i].win_ndet, delta, np, d_win + win_off[t], st) != cudaSuccess ||
-            launch_win_part(dp, i, np, rays_max, slots_of[t], longest_max, d_win + win_off[t], d_cnt + patch_off[t], nullptr, nullptr,
-                            d_err, st) != cudaSuccess)
+        if (launch_win_windows(dp, i, inst[i].win_ndet, delta, np, d_win + win_off[t], st) != cudaSuccess)
             return PAT_ERR_CUDA;
     }
+    // the samples that need a position of their own, by patch of all templates (a second
+    // pass where there are more of them than the first has room for)
+    std::vector<WinOwn> own;
+    std::vector<int> own_off(n_tmpl + 1, 0);
+    DevBuf own_buf(st);
+    WinOwn* d_own = reinterpret_cast<WinOwn*>(tb + o_own);
+    for (uint32_t cap = kOwnFirst, n = 0;; cap = n) {
+        uint32_t* d_count = reinterpret_cast<uint32_t*>(d_err) + 1;
+        if (cudaMemsetAsync(d_count, 0, sizeof(uint32_t), st) != cudaSuccess) return PAT_ERR_CUDA;
+        for (int t = 0; t < n_tmpl; ++t)
+            if (launch_win_own(dp, rep[t], inst[rep[t]].win_ndet, (int)(patch_off[t + 1] - patch_off[t]),
+                               (int)patch_off[t], d_win + win_off[t], d_own, cap, d_count, st) != cudaSuccess)
+                return PAT_ERR_CUDA;
+        if (cudaMemcpyAsync(&n, d_count, sizeof(n), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+            cudaStreamSynchronize(st) != cudaSuccess)
+            return PAT_ERR_CUDA;
+        if (n > (uint32_t)INT32_MAX) return PAT_ERR_UNSUPPORTED;
+        if (n <= cap) {
+            own.resize(n);
+            break;
+        }
+        if (!own_buf.alloc(sizeof(WinOwn) * n)) return PAT_ERR_OOM;
+        d_own = static_cast<WinOwn*>(own_buf.p);
+    }
+    if (!own.empty() &&
+        (cudaMemcpyAsync(own.data(), d_own, sizeof(WinOwn) * own.size(), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+         cudaStreamSynchronize(st) != cudaSuccess))
+        return PAT_ERR_CUDA;
+    std::sort(own.begin(), own.end(), [](const WinOwn& a, const WinOwn& b) {
+        return std::tie(a.patch, a.j, a.q, a.m) < std::tie(b.patch, b.j, b.q, b.m);
+    });
+    for (int t = 0, k = 0; t < n_tmpl; ++t) {
+        for (; k < (int)own.size() && own[k].patch < patch_off[t + 1]; ++k) own[k].patch -= (int32_t)patch_off[t];
+        own_off[t + 1] = k;
+    }
+    if (!own.empty() &&
+        cudaMemcpyAsync(d_own, own.data(), sizeof(WinOwn) * own.size(), cudaMemcpyHostToDevice, st) != cudaSuccess)
+        return PAT_ERR_CUDA;
+    auto part = [&](int t, WinBlock* blocks, WinSub* subs) {
+        return launch_win_part(dp, rep[t], (int)(patch_off[t + 1] - patch_off[t]), rays_max, slots_of[t], longest_max,
+                               d_win + win_off[t], d_own + own_off[t], own_off[t + 1] - own_off[t], d_cnt + patch_off[t],
+                               blocks, subs, d_err, st);
+    };
+    for (int t = 0; t < n_tmpl; ++t)
+        if (part(t, nullptr, nullptr) != cudaSuccess) return PAT_ERR_CUDA;
     std::vector<int4> cnt(patch_off[n_tmpl]);
     int32_t err = 0;
     if (cudaMemcpyAsync(cnt.data(), d_cnt, sizeof(int4) * cnt.size(), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
@@ -244,10 +293,9 @@ pat_status_t build_windows(Plan& P, std::vector<InstDev>& inst, const std::vecto
         cudaMemcpyAsync(d_cnt, cnt.data(), sizeof(int4) * cnt.size(), cudaMemcpyHostToDevice, st) != cudaSuccess)
         return PAT_ERR_CUDA;
     for (int t = 0; t < n_tmpl; ++t) {
-        const int i = rep[t], np = (int)(patch_off[t + 1] - patch_off[t]), nb = (int)(blk_off[t + 1] - blk_off[t]);
+        const int i = rep[t], nb = (int)(blk_off[t + 1] - blk_off[t]);
         WinBlock* tb0 = d_blocks + blk_off[t];
-        if (launch_win_part(dp, i, np, rays_max, slots_of[t], longest_max, d_win + win_off[t], d_cnt + patch_off[t], d_blocks, d_subs,
-                            d_err, st) != cudaSuccess ||
+        if (part(t, d_blocks, d_subs) != cudaSuccess ||
             launch_win_recs(dp, i, nb, tb0, d_subs, d_rays, d_slots, st) != cudaSuccess ||
             launch_win_lists(dp, i, nb, tb0, d_subs, nullptr, st) != cudaSuccess)
             return PAT_ERR_CUDA;
