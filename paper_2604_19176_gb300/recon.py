@@ -171,7 +171,7 @@ def tv_reconstruct(plan: PatPlan, g: torch.Tensor, alpha: float, eps: float = 1e
     # (ten iterations at 256^2: 1362 -> 861 us).  It reads f_k and writes the
     # other buffer: a stop at k returns f_k untouched.
     delta = [torch.empty(2 * len(plan.geoms), dtype=torch.float32, device=plan.device) for _ in range(2)]
-    sums = [torch.empty(2 * len(plan.geoms), dtype=torch.float32, pin_memory=True) for _ in range(2)]
+    sums = [torch.empty(2 * len(plan.geoms), dtype=torch.float32, device="cpu", pin_memory=True) for _ in range(2)]
     read = [torch.cuda.Event() for _ in range(2)]
     stream = torch.cuda.current_stream(plan.device)
 
