@@ -107,8 +107,9 @@ typedef struct {
     int32_t adj_mode;    /* adjoint gather: 0 = auto (windowed code lists where adj_groups    */
                          /*   and adj_jblock are 0 too, the radii that cross 8 pixels fit the */
                          /*   staged tables, the codes the list budget, and the plan has 600  */
-                         /*   patches of 8 x 8 pixels or some 12 M samples; else 4 if it fits */
-                         /*   the budget, else 1, else 3, else 2);                            */
+                         /*   patches of 8 x 8 pixels or some 12 M samples (3800 patches if   */
+                         /*   no images share lists and many detectors lie around the image); */
+                         /*   else 4 if it fits the budget, else 1, else 3, else 2);          */
                          /*   1 = per-cell sample code lists built at                         */
                          /*   creation (device memory ~4 B per sample); 2 = enumerate on      */
                          /*   every call (no list memory); 3 = per-cell fraction lists built  */

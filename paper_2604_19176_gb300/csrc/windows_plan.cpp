@@ -98,6 +98,38 @@ int32_t win_symmetry(const pat_geometry_t& g, int max_order)
     return ring && g.n_angles % 2 == 0 ? kSymHalf : kSymNone;
 }
 
+// Images that share lists are fewer, longer pieces of work: as many together
+// as leave every resident warp two blocks of 64 rays (adjoint at 128^2, 64
+// detectors: 19 us single, 21.5 us in pairs; at 256^2, 128 detectors: 42 us
+// single, 36 us in pairs).
+int images_together(const pat_geometry_t* geoms, int n_inst, double warps)
+{
+    double rays = 0.0;
+    for (int i = 0; i < n_inst; ++i) rays += kPatchRays * patches_of(geoms[i].n) * patches_of(geoms[i].n) * geoms[i].n_det;
+    int nb = 4;
+    while (nb > 1 && rays / nb < 2.0 * 64.0 * warps) nb /= 2;
+    return nb;
+}
+
+bool same_geometry(const pat_geometry_t& a, const pat_geometry_t& b)
+{
+    return a.n == b.n && a.n_det == b.n_det && a.arc_start == b.arc_start && a.arc_span == b.arc_span &&
+           a.n_t == b.n_t && a.t_max == b.t_max && a.n_angles == b.n_angles;
+}
+
+// Whether any two images of a plan share lists: those of one symmetric
+// geometry or of two equal ones.
+bool share_lists(const pat_geometry_t* geoms, int n_inst, int nb_max)
+{
+    if (nb_max < 2) return false;
+    for (int i = 0; i < n_inst; ++i) {
+        if (win_symmetry(geoms[i], nb_max) != kSymNone) return true;
+        for (int k = 0; k < i; ++k)
+            if (same_geometry(geoms[i], geoms[k])) return true;
+    }
+    return false;
+}
+
 } // namespace
 
 bool windows_fit(const pat_geometry_t* geoms, int n_inst, int num_sms)
@@ -121,6 +153,27 @@ bool windows_fit(const pat_geometry_t* geoms, int n_inst, int num_sms)
     // with 320 detectors, 70.6 / 47.3 for 128^2 with 512) the windows win.
     const double warps = 20.0 * num_sms;
     if (patches < warps / 5.0 && samples < 4000.0 * warps) return false;
+    // Lists that serve one image each cost twice as much per sample as shared
+    // ones.  Where, besides, the detectors lie all around the image, the cells'
+    // lists are about equally long (the per-cell form's weakness is the crowd of
+    // a short arc), and with many detectors and not too many patches the
+    // per-cell lists are faster.  Measured over 400 drawn geometries on arcs of
+    // 185 degrees and more, per-cell / windows: 0.79 to 1.02, mostly 0.85 to
+    // 0.95, below 1064 patches from 0.4 detectors per pixel column on (46 / 52
+    // us for 176^2 with 292 detectors on 200 degrees), and 0.82 to 1.05 below
+    // 3800 from 0.7 on (216 / 249 us for 476^2 with 391 on 309 degrees).
+    // Outside: 1.04 to 1.35 at 3800 to 4500 patches (418 / 491 us for 512^2
+    // with 511 on a ring over windows / per cell), 1.0 to 1.3 with few
+    // detectors, 1.2 to 1.9 on half a ring and less.
+    if (patches < 1.25 * warps && !share_lists(geoms, n_inst, images_together(geoms, n_inst, warps))) {
+        const double half_turn = 3.14159265358979323846;
+        const bool few = patches < 0.35 * warps;
+        bool around = true;
+        for (int i = 0; i < n_inst; ++i)
+            around = around && geoms[i].arc_span > (few ? 1.1 : 1.3) * half_turn &&
+                     geoms[i].n_det > (few ? 0.4 : 0.7) * geoms[i].n;
+        if (around) return false;
+    }
     return windows * sizeof(int4) <= 4e9;   // (build-time table)
 }
 
@@ -131,18 +184,11 @@ pat_status_t build_windows(Plan& P, std::vector<InstDev>& inst, const std::vecto
     const int n_inst = (int)inst.size();
     const int64_t warps = (int64_t)std::max(1, adj_win_blocks_per_sm(1)) * P.num_sms * (kWinThreads / kWarp);
     std::vector<int> rep(n_tmpl, -1);
-    double rays_all = 0.0;
     for (int i = 0; i < n_inst; ++i) {
         if (rep[inst_tmpl[i]] < 0) rep[inst_tmpl[i]] = i;
         inst[i].win_px = patches_of(inst[i].n);
-        rays_all += kPatchRays * inst[i].win_px * inst[i].win_px * inst[i].n_det;
     }
-    // Images that share lists are fewer, longer pieces of work: as many
-    // together as leave every resident warp two blocks of 64 rays.
-    // (adjoint at 128^2, 64 detectors: 19 us single, 21.5 us in pairs; at
-    // 256^2, 128 detectors: 42 us single, 36 us in pairs)
-    int nb_max = 4;
-    while (nb_max > 1 && rays_all / nb_max < 2.0 * 64.0 * (double)warps) nb_max /= 2;
+    const int nb_max = images_together(P.geoms.data(), n_inst, (double)warps);
     for (int i = 0; i < n_inst; ++i) {
         inst[i].win_sym = win_symmetry(P.geoms[i], nb_max);
         inst[i].win_ndet = inst[i].n_det / win_sym_order(inst[i].win_sym);
