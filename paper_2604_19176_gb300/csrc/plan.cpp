@@ -6,6 +6,7 @@
 #include <cstring>
 #include <map>
 #include <mutex>
+#include <new>
 #include <numeric>
 #include <queue>
 #include <thread>
@@ -226,8 +227,12 @@ void choose_tile(int n, int64_t cells, int want_w, int want_h, int& tw, int& th)
 static_assert(sizeof(InstDev) % 8 == 0, "InstDev layout");
 static_assert(sizeof(Unit) == 32, "Unit layout");
 
-pat_status_t build_plan(Plan& P, const pat_geometry_t* geoms, int n_inst, const pat_options_t& opt,
-                        cudaStream_t st)
+namespace {
+
+// build_plan with the windowed lists allowed or not; windows_failed: they were
+// chosen and there was no room for them.
+pat_status_t build_plan_form(Plan& P, const pat_geometry_t* geoms, int n_inst, const pat_options_t& opt,
+                             cudaStream_t st, bool windows, bool& windows_failed)
 {
     P.n_inst = n_inst;
     P.geoms.assign(geoms, geoms + n_inst);
@@ -313,7 +318,7 @@ pat_status_t build_plan(Plan& P, const pat_geometry_t* geoms, int n_inst, const 
     std::vector<float2> rtrig;
     // windowed adjoint lists (windows.cu), the default where their staged
     // tables hold a patch's radii: detectors and directions in fixed point
-    const bool win_wanted = opt.adj_mode == 0 && opt.adj_groups == 0 && opt.adj_jblock == 0 &&
+    const bool win_wanted = windows && opt.adj_mode == 0 && opt.adj_groups == 0 && opt.adj_jblock == 0 &&
                             windows_fit(geoms, n_inst, P.num_sms);
     std::vector<int4> win_det;
     std::vector<uint4> win_dirs;
@@ -1029,8 +1034,14 @@ pat_status_t build_plan(Plan& P, const pat_geometry_t* geoms, int n_inst, const 
     int64_t list_bytes = 0;
     if (use_win) {
         int parts = 1;
-        const pat_status_t s = build_windows(P, inst, inst_tmpl, (int)tmpls.size(),
-                                             reinterpret_cast<InstDev*>(base + o_inst), &list_bytes, &parts, st);
+        pat_status_t s;
+        try {
+            s = build_windows(P, inst, inst_tmpl, (int)tmpls.size(), reinterpret_cast<InstDev*>(base + o_inst),
+                              &list_bytes, &parts, st);
+        } catch (const std::bad_alloc&) {
+            s = PAT_ERR_OOM;
+        }
+        windows_failed = s == PAT_ERR_OOM || s == PAT_ERR_UNSUPPORTED;
         if (s != PAT_OK) return s;
         dp.adj_groups = parts;
     }
@@ -1360,9 +1371,21 @@ pat_status_t build_plan(Plan& P, const pat_geometry_t* geoms, int n_inst, const 
     return PAT_OK;
 }
 
-namespace {
 std::atomic<int32_t> g_alloc_fail{-1};   // see set_alloc_failure
 } // namespace
+
+// The windowed lists take up to twice the memory of the per-cell ones while
+// they are built (6.9 and 3.3 GB for 2048^2, 3000 detectors and 64 angles), so
+// a plan that has no room for them is built over those.
+pat_status_t build_plan(Plan& P, const pat_geometry_t* geoms, int n_inst, const pat_options_t& opt, cudaStream_t st)
+{
+    bool windows_failed = false;
+    const pat_status_t s = build_plan_form(P, geoms, n_inst, opt, st, true, windows_failed);
+    if (!windows_failed) return s;
+    free_plan_memory(P);
+    P = Plan();
+    return build_plan_form(P, geoms, n_inst, opt, st, false, windows_failed);
+}
 
 void set_alloc_failure(int32_t n) { g_alloc_fail.store(n < 0 ? -1 : n); }
 
