@@ -152,8 +152,8 @@ typedef struct {
     int32_t tile_cols;       /* widest circular-mean tile (pixels); band_rows the tallest */
     int32_t time_pair;       /* 1 = the steps run the fused time stage, 0 = separate      */
     int32_t adj_jblock;      /* detectors per aligned block of the code lists (0: none)   */
-    int32_t adj_windows;     /* 1 = the code lists are in windowed form (adj_mode then    */
-                             /*   gives the form that the geometry's codes would take)    */
+    int32_t adj_windows;     /* 1 = the lists are windowed (adj_mode then gives the form  */
+                             /*   that an automatic plan would take without windows)      */
 } pat_plan_info_t;
 
 /*

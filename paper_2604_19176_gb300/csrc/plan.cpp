@@ -1359,7 +1359,7 @@ pat_status_t build_plan_form(Plan& P, const pat_geometry_t* geoms, int n_inst, c
             I.tile_cols = std::max(I.tile_cols, t.x1 - t.x0);
         }
     I.adj_groups = dp.adj_groups;
-    I.adj_mode = use_win ? (pairs_fit ? 4 : 1) : dp.adj_mode == 0 ? 2 : dp.adj_mode;
+    I.adj_mode = use_win ? list_mode : dp.adj_mode == 0 ? 2 : dp.adj_mode;
     I.adj_windows = use_win ? 1 : 0;
     I.abel_split_fwd = dp.abel_cluster_fwd;
     I.abel_split_adj = dp.abel_cluster_adj;
