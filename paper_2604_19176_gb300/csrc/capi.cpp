@@ -255,12 +255,8 @@ pat_status_t pat_forward(pat_plan_t h, const void* d_f, float* d_g, void* stream
     DeviceScope ds(p->device);
     if (!ds.ok) return PAT_ERR_CUDA;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    // radius sums and time stage in one launch where the steps fuse them too
-    const bool fused = p->dp.time_chunks > 0;
-    cudaError_t e = timed(*p, PAT_K_CIRCMEAN, st, [&] { return circmean(*p, d_f, st, !fused); });
-    if (e == cudaSuccess)
-        e = timed(*p, PAT_K_ABEL_FWD, st,
-                  [&] { return fused ? launch_time_fwd(p->dp, d_g, st) : launch_abel_fwd(p->dp, d_g, st); });
+    cudaError_t e = timed(*p, PAT_K_CIRCMEAN, st, [&] { return circmean(*p, d_f, st, forward_msum(p->dp)); });
+    if (e == cudaSuccess) e = timed(*p, PAT_K_ABEL_FWD, st, [&] { return launch_forward_time(p->dp, d_g, st); });
     return cuda_status(e);
 }
 

@@ -48,6 +48,14 @@ cudaError_t launch_time_pair(const DevPlan& dp, const float* g, float* y, bool d
                              cudaStream_t st);
 // Its forward half alone (radius sums and forward): g = A f from the partial slots.
 cudaError_t launch_time_fwd(const DevPlan& dp, float* g, cudaStream_t st);
+// What pat_forward runs after the circular means: radius sums and time stage in
+// one launch on the plans whose steps fuse theirs (the circular-mean launch is
+// then without its radius sums: forward_msum), else the separate time stage.
+inline bool forward_msum(const DevPlan& dp) { return dp.time_chunks <= 0; }
+inline cudaError_t launch_forward_time(const DevPlan& dp, float* g, cudaStream_t st)
+{
+    return forward_msum(dp) ? launch_abel_fwd(dp, g, st) : launch_time_fwd(dp, g, st);
+}
 // Clusters of the fused time stage that fit the GPU at once (0: cannot run).
 int time_pair_clusters(int smem_bytes);
 cudaError_t launch_adjoint_gather(const DevPlan& dp, void* f, cudaStream_t st);

@@ -181,9 +181,9 @@ pat_status_t autotune_plan(Plan** out, const pat_geometry_t* geoms, int n_inst, 
                 o.adj_groups = 1;
                 Plan* p = try_build(geoms, n_inst, o, st);
                 if (!p) continue;
-                const float ms = time_ms(st, 2, 5, [&] {
-                    cudaError_t e = launch_circmean(p->dp, d_f, st);
-                    return e == cudaSuccess ? launch_abel_fwd(p->dp, d_g, st) : e;
+                const float ms = time_ms(st, 2, 5, [&] {   // (the launches of pat_forward)
+                    cudaError_t e = launch_circmean(p->dp, d_f, st, forward_msum(p->dp));
+                    return e == cudaSuccess ? launch_forward_time(p->dp, d_g, st) : e;
                 });
                 drop(p);
                 if (ms > 0.f && ms < best_ms) {
@@ -202,8 +202,8 @@ pat_status_t autotune_plan(Plan** out, const pat_geometry_t* geoms, int n_inst, 
             o.abel_split = cs;
             Plan* p = try_build(geoms, n_inst, o, st);
             if (!p) continue;
-            const float ms = time_ms(st, 2, 5, [&] {
-                cudaError_t e = launch_abel_fwd(p->dp, d_g, st);
+            const float ms = time_ms(st, 2, 5, [&] {   // (where the forward's is fused it has no split)
+                cudaError_t e = forward_msum(p->dp) ? launch_abel_fwd(p->dp, d_g, st) : cudaSuccess;
                 return e == cudaSuccess ? launch_abel_adj(p->dp, d_g, st) : e;
             });
             drop(p);
