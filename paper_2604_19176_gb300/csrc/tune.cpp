@@ -48,6 +48,7 @@ std::string tune_key(const pat_geometry_t* geoms, int n, const pat_options_t& op
     put(&opt.adj_mode, sizeof opt.adj_mode);
     put(&opt.time_pair, sizeof opt.time_pair);
     put(&opt.adj_jblock, sizeof opt.adj_jblock);
+    put(&opt.adj_groups, sizeof opt.adj_groups);   // (given: no windowed lists)
     put(&device, sizeof device);
     return k;
 }

@@ -22,6 +22,7 @@ pat_status_t build_plan(Plan& P, const pat_geometry_t*, int, const pat_options_t
     std::printf("build mode=%d split=%d\n", (int)opt.adj_mode, (int)opt.abel_split);
     P.opt = opt;
     P.dp.time_chunks = g_chunks;
+    P.info.adj_windows = opt.adj_mode == 0 && opt.adj_groups == 0 && opt.adj_jblock == 0;
     return PAT_OK;
 }
 void free_plan_memory(Plan&) {}
@@ -57,8 +58,14 @@ int main(int, char** a)
     pat_geometry_t g{64, 16, 0.0, 3.0, 64, 2.0, 64};
     pat_options_t opt{};
     opt.tune = 1;
-    Plan* p = nullptr;
-    return autotune_plan(&p, &g, 1, opt, nullptr) == PAT_OK && p ? 0 : 1;
+    for (int i = 2; a[i]; ++i) {
+        opt.adj_groups = atoi(a[i]);
+        std::printf("call groups=%d\n", (int)opt.adj_groups);
+        Plan* p = nullptr;
+        if (autotune_plan(&p, &g, 1, opt, nullptr) != PAT_OK || !p) return 1;
+        std::printf("plan windows=%d\n", (int)p->info.adj_windows);
+    }
+    return 0;
 }
 """
 
@@ -76,14 +83,17 @@ def program(tmp_path_factory):
     return str(exe)
 
 
+def _run(program, *args):
+    return subprocess.run([program, *map(str, args)], check=True, capture_output=True, text=True).stdout.splitlines()
+
+
 @pytest.mark.parametrize("chunks,forward,split", [
     (2, ["circmean msum=0", "time_fwd"], ["abel_adj"]),                  # fused time stage, as pat_forward runs it
     (0, ["circmean msum=1", "abel_fwd"], ["abel_fwd", "abel_adj"]),      # separate
 ])
 def test_timed_launches(program, chunks, forward, split):
-    lines = subprocess.run([program, str(chunks)], check=True, capture_output=True, text=True).stdout.splitlines()
     plans, launches = [], None
-    for x in lines:
+    for x in _run(program, chunks, 0)[1:-1]:
         if x.startswith("build"):
             launches = []
             plans.append((x, launches))
@@ -97,3 +107,12 @@ def test_timed_launches(program, chunks, forward, split):
     assert len(fwd) >= 3 and all(r == forward * 7 for r in fwd)          # 2 warm and 5 timed calls
     assert len(splits) == 4 and all(r == split * 7 for r in splits)
     assert adjoint and all(r == ["abel_adj", "gather"] * 7 for r in adjoint)
+
+
+@pytest.mark.parametrize("calls", [(0, 4, 0), (4, 0, 4)])
+def test_list_parts_asked_for_are_not_answered_from_the_cache(program, calls):
+    """A request for a number of list parts never takes the windowed lists, also when an automatic plan of the same
+    geometry was tuned before, and the other way round."""
+    lines = [x for x in _run(program, 2, *calls) if x.startswith(("call", "plan"))]
+    # (the stand-in's candidates all take the same time: an automatic plan keeps its first, the windowed one)
+    assert lines == [x for c in calls for x in (f"call groups={c}", f"plan windows={int(c == 0)}")]
