@@ -348,8 +348,10 @@ pat_status_t pat_plan_set_wait_probe(pat_plan_t plan, int32_t clocks);
  * != 0, the next adjoint gather of this plan (pat_adjoint, pat_tv_step,
  * pat_pdhg_step) in code- or fraction-list form gives the first entry of its
  * first warp's first item a detector index (and Mbar index) past the
- * instance's detectors; everything that index would address still lies inside
- * the plan's allocations, so nothing faults even where a check were missing.
+ * instance's detectors (windowed lists: the first entry of every CTA a radius
+ * past its staged ones); everything that index would address still lies inside
+ * the plan's allocations (the CTA's shared memory), so nothing faults even
+ * where a check were missing.
  * The entry check reports it and the entry is skipped.  The probe disarms
  * itself after that one launch.  Returns PAT_ERR_UNSUPPORTED in release
  * builds.  Synchronous with respect to the host only.

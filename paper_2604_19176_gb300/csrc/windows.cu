@@ -151,7 +151,8 @@ __host__ __device__ constexpr int win_warp_bytes(int nb)
     return win_rays(nb) * 16 + win_slots(nb) * 4 * nb;
 }
 static_assert(win_warp_bytes(1) % kWinAlign == 0 && win_warp_bytes(2) % kWinAlign == 0 &&
-                  win_warp_bytes(4) % kWinAlign == 0 && win_rays(1) * 16 <= (int)kWinAlign,
+                  win_warp_bytes(4) % kWinAlign == 0 && win_rays(1) * 16 <= (int)kWinAlign &&
+                  win_slots(1) * 4 <= 0x1400 && win_slots(2) * 4 <= 0x1400 && win_slots(4) * 4 <= 0x1400,
               "staged tables of a warp");
 
 __device__ __forceinline__ uint4 lds128(uint32_t addr)
@@ -229,7 +230,7 @@ __global__ void __launch_bounds__(kWinThreads, NB == 4 ? 4 : 5)
     };
     clear_totals();
 #ifdef PAT_DEBUG
-    bool plant = dp.bounds_probe != 0 && blockIdx.x == 0 && share0 == 0 && threadIdx.x == 0;
+    bool plant = dp.bounds_probe != 0 && share0 == 0 && threadIdx.x == 0;   // (in every CTA: some warps have no entries)
 #endif
     int ticket = wid;
     for (int k = 0; k < sh.count; ++k) {
@@ -306,7 +307,7 @@ __global__ void __launch_bounds__(kWinThreads, NB == 4 ? 4 : 5)
             uint32_t mo = c >> 16, ro = c & (kWinAlign - 16u);
 #ifdef PAT_DEBUG
             if (plant) {
-                mo += 0x8000u;
+                mo += 0x1400u;   // past the radii of any form, inside the CTA's shared memory
                 plant = false;
             }
             // (an entry out of bounds is given the null entry's place)
