@@ -162,7 +162,6 @@ struct GeomTemplate {
 };
 
 constexpr double kStageCost = 60.0;    // staging a tile, in angle iterations of each warp (30 to 150: within 1 %)
-constexpr int kUnitsPerWarp = 1;       // units per warp from which on a plan uses more CTAs
 constexpr double kUnitOverhead = 3.0;  // per-unit fixed cost, in angle iterations (at 10: 3 % slower at 1024^2)
 // An angle iteration of a plan with radius steps of `delta` pixels, relative to
 // one of fine steps: the further apart the radii of neighbouring lanes, the
@@ -610,7 +609,7 @@ pat_status_t build_plan_form(Plan& P, const pat_geometry_t* geoms, int n_inst, c
                 n_units_all += (int64_t)tt.units.size();
             }
     const int n_ctas = (int)std::max<int64_t>(
-        1, std::min<int64_t>(n_ctas_target, n_units_all / (warps_cta * kUnitsPerWarp)));
+        1, std::min<int64_t>(n_ctas_target, n_units_all / warps_cta));   // (a unit for every warp)
     // cut(T, emit): the shares of at most T, in order; returns their number.  A
     // tile's last units join a share that they exceed by less than 0.03 T, and
     // no share takes less than 0.05 T of a tile.
