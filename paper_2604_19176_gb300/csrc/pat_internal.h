@@ -196,8 +196,10 @@ struct WinBlock {
 // radius mc (list building only).  own: only the sample (q0, mc) of them, one
 // that the patch's window of detector j cannot hold (win_position.h).
 struct WinSub {
-    int32_t j, q0, nq, m0, nm, mc, own;
+    int32_t j, q0;
+    uint16_t nq, nm, m0, mc;       // (a block's rays; a patch's radii; n_t + 2 <= 16386)
     uint16_t ray0, slot0;
+    int32_t own;
 };
 
 // Such a sample: its patch, detector, angle and radius.

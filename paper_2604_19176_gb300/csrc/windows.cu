@@ -623,7 +623,9 @@ __global__ void k_win_part(DevPlan dp, int inst_idx, int patches, int max_rays, 
             slots = 8;
             sub_first = ns;
         }
-        if (subs) subs[base.y + ns] = {j, q0, n, m0, nm, mc, own_sample, (uint16_t)rays, (uint16_t)slots};
+        if (subs)
+            subs[base.y + ns] = {j, q0, (uint16_t)n, (uint16_t)nm, (uint16_t)m0, (uint16_t)mc, (uint16_t)rays, (uint16_t)slots,
+                                 own_sample};
         rays += n4;
         slots += nmp;
         longest += len;
