@@ -796,7 +796,7 @@ def main():
                        "copied out, per step",
                "separate_calls": {"value": job_value(em_sep, world), "ms_per_step": em_sep,
                                   "note": "the same copies around pat_forward(f) and pat_adjoint(g) as two calls "
-                                          "(no fused time stage)"}}
+                                          "(the time stages of A and A^T in launches of their own)"}}
 
     cpu = None
     if rank == 0 and world == 1 and not args.no_cpu_baseline and not args.profile:

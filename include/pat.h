@@ -118,7 +118,8 @@ typedef struct {
                          /*   pair of samples at consecutive radii of one ray, or per lone    */
                          /*   sample; needs one code bit more than 1)                         */
     int32_t abel_split;  /* CTAs (a thread-block cluster) sharing each time-stage tile: 1, 2, */
-                         /*   4 or 8; 0 = auto (more when there are fewer tiles than SMs)     */
+                         /*   4 or 8; 0 = auto (more the fewer tiles there are: up to 3.5     */
+                         /*   CTAs per SM of 64 x 64 tiles, 2 per SM of 32 x 32 ones)         */
     int32_t tile_cols;   /* max pixel columns of a circular-mean tile; 0 = auto               */
     int32_t time_pair;   /* time stages of pat_tv_step / pat_pdhg_step: 0 = auto (one fused   */
                          /*   launch per step on plans of up to about 25 M time multiply-adds */
@@ -364,8 +365,9 @@ pat_status_t pat_plan_set_bounds_probe(pat_plan_t plan, int32_t enable);
  * pat_plan_create (any build).  After pat_debug_fail_alloc(n), the n-th next
  * device allocation made by plan creation or by the autotuner (n = 0: the
  * next one) fails as if the device were out of memory, once; the call that
- * made it then returns PAT_ERR_OOM (an autotuner candidate that fails is
- * skipped instead) after freeing every allocation it had made.  n < 0
+ * made it then returns PAT_ERR_OOM after freeing every allocation it had made
+ * (instead, an autotuner candidate that fails is skipped, and a plan whose
+ * windowed lists fail is built over the per-cell ones).  n < 0
  * disarms the hook.  Process-wide, for all devices; always returns PAT_OK.
  */
 pat_status_t pat_debug_fail_alloc(int32_t n);

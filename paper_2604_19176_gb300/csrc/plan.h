@@ -44,14 +44,14 @@ struct Plan {
 };
 
 // Builds all tables, schedules and tiles of P for the given geometries and
-// (already defaulted and validated) options; uploads them on `st` and waits.
+// (already validated) options; uploads them on `st` and waits.
 pat_status_t build_plan(Plan& P, const pat_geometry_t* geoms, int n_inst, const pat_options_t& opt,
                         cudaStream_t st);
 void free_plan_memory(Plan& P);
 
 // Windowed adjoint lists (windows_plan.cpp).  windows_fit: whether the staged
-// tables hold every geometry's windows, and the plan has enough work for them.  build_windows builds them for the
-// plan's instances (inst_tmpl: the geometry template of each) on `st`, fills
+// tables hold every geometry's windows, and the lists are the faster form for
+// such a plan.  build_windows builds them for the plan's instances (inst_tmpl: the geometry template of each) on `st`, fills
 // dp.win_* and the instances' fields (uploaded to d_inst), and gives the
 // device bytes and the most parts a patch is split into.
 bool windows_fit(const pat_geometry_t* geoms, int n_inst, int num_sms);

@@ -165,6 +165,9 @@ bool windows_fit(const pat_geometry_t* geoms, int n_inst, int num_sms)
     // Outside: 1.04 to 1.35 at 3800 to 4500 patches (418 / 491 us for 512^2
     // with 511 on a ring over windows / per cell), 1.0 to 1.3 with few
     // detectors, 1.2 to 1.9 on half a ring and less.
+    // (Both forms are far inside the 1e-5 bound: 2e-7 to 6e-7 of the image per
+    // cell, whose sums are one chain, 1.3e-7 to 1.7e-7 over windows, for bipolar
+    // pulses with 1 % noise.)
     if (patches < 1.25 * warps && !share_lists(geoms, n_inst, images_together(geoms, n_inst, warps))) {
         const double half_turn = 3.14159265358979323846;
         const bool few = patches < 0.35 * warps;
